@@ -24,6 +24,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "ts_emu.h"
 #include "ts_internal.h"
 
 using ts::Dims;
@@ -582,6 +583,7 @@ ts::Problem make_problem(const ts_grid* g) {
   p.op64 = g->t64.OpT;
   p.mc64 = g->t64.DrMc;
   p.tcang = g->tcang;
+  p.emu = g->emu;
   if (g->sn > 0) {   // one slice of groups: every per-group pointer offset to group s0
     const long long per = g->d.nblk / g->d.G;
     const long long infl = (long long)g->d.Nt * g->d.Np * (g->d.NT / 2) * g->d.NP;
@@ -1116,6 +1118,10 @@ ts_status ts_create_grid(const ts_grid_desc* desc, ts_grid** out) {
     if (e == cudaSuccess)
       e = cudaMemcpy(G->tcb16, b16.data(), b16.size() * sizeof(uint16_t), cudaMemcpyHostToDevice);
   }
+  if (e == cudaSuccess && g.precision == TS_FP64) {
+    const char* gen = std::getenv("TS_GENERIC_PASSES");
+    if (!gen || gen[0] != '1') G->emu = ts::emu_create(g, &e);
+  }
   const size_t ncoef = (size_t)d.nblk * sizeof(double);
   const size_t ninfl = (size_t)g.groups * g.Ntheta * g.Nphi * (g.NTheta / 2) * g.NPhi * es;
   const size_t nf = (size_t)d.total * es;
@@ -1172,6 +1178,7 @@ ts_status ts_destroy_grid(ts_grid* g) {
   for (void* p : g->adj)
     if (p) cudaFree(p);
   if (g->piw) cudaFree(g->piw);
+  ts::emu_destroy(g->emu);
   for (cudaEvent_t e : g->ev) cudaEventDestroy(e);
   if (g->cs_in) cudaStreamDestroy(g->cs_in);
   if (g->cs_out) cudaStreamDestroy(g->cs_out);

@@ -134,6 +134,7 @@ void tune_store_locked(const std::string& key, const TileParams& tp) {
 template <typename T, typename C>
 cudaError_t tune_grid(ts_grid* g, const Tables<C>& t, cudaStream_t st, TileParams* out) {
   Problem p = problem_of(g);
+  p.emu = nullptr;   // tile shapes are those of the passes on the FP64 (FP32) units
   const Dims& d = p.d;
   T* U = static_cast<T*>(g->U);
   T* K = static_cast<T*>(g->K);

@@ -38,6 +38,7 @@
 // group's blocks in a fixed order.
 #include <algorithm>
 
+#include "ts_emu.h"
 #include "ts_internal.h"
 
 namespace ts {
@@ -371,6 +372,10 @@ k_balance_groups(const double* __restrict__ part, long long per, double* __restr
 template <typename T>
 cudaError_t launch_angular_cons(const Problem& p, const Tables<T>& t, const T* U, T* K, T sgn,
                                 bool collision, cudaStream_t s) {
+  if constexpr (sizeof(T) == 8) {
+    if (p.emu && emu_has_angular(*p.emu, p.d))
+      return emu_angular(*p.emu, p, t, true, U, K, sgn, collision, s);
+  }
   const ConsTile c = cons_tile(p.d, sizeof(T));
   cudaError_t e = cudaFuncSetAttribute(k_angular_cons<T>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.bytes);

@@ -1,0 +1,1216 @@
+// Double-precision contractions on the 5th-generation tensor cores.
+//
+// GB300 issues 2 FP64 multiply-adds per SM and clock, against 4096 f16 products:
+// the FP64 pipe bounds every double-precision pass that contracts on it. Here the
+// contractions run as exact integer arithmetic on tcgen05.mma kind::f16:
+//  * data: a tile's values are turned into 64-bit fixed point relative to the
+//    largest magnitude of a block (61 bits below it), on the integer units, and
+//    cut into eight bytes u_i. A byte zero-extended to 16 bits is the f16
+//    subnormal u_i 2^-24, so the digits need no conversion. Balanced digits are
+//    d_i = u_i - 128 (the fixed-point value has 0x8080...80 added);
+//  * matrix: every row scaled to 62 bits, in eight balanced base-256 digits e_j as
+//    f16 integers (built on the host from the exact products of its factors);
+//  * the products d_i e_j of order o = i + j <= 7 are accumulated in f32, one
+//    tensor-memory column per output and order: multiples of 2^-24 that stay below
+//    2^22 units (checked on the host), so every accumulation is exact. One MMA per
+//    digit i covers all e_j (N = outputs x (8 - i), accumulator columns shifted by
+//    i x outputs). A first MMA sets every accumulator to 0.75 - 128 sum e_j
+//    2^-24: it removes the byte offset, and the accumulator's bit pattern is then
+//    0x3F400000 + (the exact integer sum);
+//  * the eight sums are recombined in a 64-bit integer (orders >= 8, 2^-59 of the
+//    full scale, are dropped) and rounded once to double on the integer units.
+// The error of a contraction is that one rounding, less than that of the FP64
+// multiply-adds it replaces: against the operator in extended precision one right-hand
+// side is 1.2e-15 (17 x 8^4), 6.1e-15 (33 x 8^4), 7.9e-16 (9 x 16^2 x 8^2) off in the
+// relative 2-norm where the FP64 passes are 2.0e-14, 2.6e-14 and 1.5e-14 off. A block that
+// holds an infinity or a NaN gives NaN.
+//
+// What bounds the passes now: the integer instructions that cut, recombine and round
+// (about 240 a point and pass, 64-bit multiplies among them), at 1.5 instructions per
+// clock from 16 warps an SM; tensor pipe 9 %, FP64 pipe 20-40 %, HBM 10-15 % busy.
+//
+// Every wait is bounded: if one runs out the kernel sets the grid's error flag
+// (ts_sync_status reports TS_ERR_TIMEOUT), waits again for its own MMAs, frees its
+// tensor memory and returns.
+#pragma once
+
+#include <stdint.h>
+
+#include "ts_emu.h"
+#include "ts_kernels.cuh"
+
+namespace ts {
+namespace emu {
+
+constexpr uint32_t kMagic = 0x3F400000u;   // bits of 0.75f
+
+__device__ __forceinline__ uint32_t sm_u32(const void* p) {
+  return (uint32_t)__cvta_generic_to_shared(p);
+}
+
+__device__ __forceinline__ bool bar_wait(uint32_t addr, uint32_t parity, long long iters) {
+  for (long long it = 0; it < iters; ++it) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok) : "r"(addr), "r"(parity) : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+
+// Shared-memory matrix descriptors, no swizzle. K-major operand (8-row x 16-byte
+// cores): lbo the distance of cores along K, sbo of 8-row groups. MN-major operand
+// (cores of 8 K x 8 rows, rows fastest): lbo the distance of 8-deep K groups, sbo of
+// 8-row groups. Low word: address and lbo in 16-byte units; high word: sbo, version.
+
+// One MMA chain step: D[128 x N] += A B. Called by a whole warp with warp-uniform
+// arguments, `one` set on the elected lane: operands in uniform registers issue an
+// MMA every 62 clocks, against 163 from a divergent branch of one thread. The
+// descriptors come in halves: the high words do not change along a chain.
+__device__ __forceinline__ uint32_t idesc_f16(int N, bool a_mn) {
+  return (1u << 4) | (a_mn ? 1u << 15 : 0u) | ((uint32_t)(N >> 3) << 17) |
+         ((uint32_t)(128 >> 4) << 24);
+}
+__device__ __forceinline__ void mma_f16(uint32_t one, uint32_t d, uint32_t alo, uint32_t ahi,
+                                        uint32_t blo, uint32_t bhi, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p, q;\n .reg .b64 a, b;\n setp.ne.b32 p, %6, 0;\n"
+      " setp.ne.b32 q, %7, 0;\n mov.b64 a, {%1, %2};\n mov.b64 b, {%3, %4};\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n}\n"
+      :: "r"(d), "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(acc), "r"(one)
+      : "memory");
+}
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr, uint32_t lbo) {
+  return (saddr >> 4) | ((lbo >> 4) << 16);
+}
+__device__ __forceinline__ uint32_t desc_hi(uint32_t sbo) { return (sbo >> 4) | (1u << 14); }
+
+// The chain of one accumulator tile: the bias step, then for every digit i and K
+// step the products with the matrix digits j <= 7 - i. a: digit 0 of the rows (MN-
+// major, digit stride ad, row-group stride asbo); K steps: OWN pairs of K cores of
+// the line, the same of the partner `part` bytes on (PART), then (ODD) one step of
+// the line's and the partner's last cores. b: the matrix (bias core, `skip` more
+// cores, K cores), `rows` rows a core; n outputs. Unrolled: an MMA then issues every
+// 50 clocks, against 153 from run-time loops over digits and K steps.
+template <int OWN, bool PART, bool ODD>
+__device__ __forceinline__ void chain_steps(uint32_t one, uint32_t tm, uint32_t bias, uint32_t a,
+                                            uint32_t ad, uint32_t asbo, uint32_t part, uint32_t b,
+                                            int skip, int rows, int n) {
+  const uint32_t core = (uint32_t)rows;   // 16-byte units
+  const uint32_t bhi = desc_hi(128), ahi = desc_hi(asbo);
+  const uint32_t b0 = desc_lo(b, core * 16u), bk = b0 + core * (uint32_t)(1 + skip);
+  const uint32_t a0 = desc_lo(a, 128);
+  mma_f16(one, tm, desc_lo(bias, 2048), desc_hi(128), b0, bhi, idesc_f16((8 * n + 15) & ~15, false),
+          0);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const uint32_t id = idesc_f16(((8 - i) * n + 15) & ~15, true);
+    const uint32_t d = tm + (uint32_t)(i * n), al = a0 + (uint32_t)i * (ad >> 4);
+#pragma unroll
+    for (int ks = 0; ks < OWN; ++ks)
+      mma_f16(one, d, al + 16u * ks, ahi, bk + 2 * core * ks, bhi, id, 1);
+    if (PART) {
+#pragma unroll
+      for (int ks = 0; ks < OWN; ++ks)
+        mma_f16(one, d, al + (part >> 4) + 16u * ks, ahi, bk + 2 * core * (OWN + ks), bhi, id, 1);
+      if (ODD)
+        mma_f16(one, d, (al & 0xFFFFu) + 16u * OWN + ((part >> 4) << 16), ahi, bk + 4 * core * OWN,
+                bhi, id, 1);
+    }
+  }
+}
+// The same with run-time K steps, and column blocks of 256 for wider accumulators.
+__device__ __noinline__ void chain_any(uint32_t one, uint32_t tm, uint32_t bias, uint32_t a,
+                                       uint32_t ad, uint32_t asbo, int own, uint32_t part, bool odd,
+                                       uint32_t b, int skip, int rows, int n) {
+  const uint32_t core = (uint32_t)rows;
+  const uint32_t bhi = desc_hi(128), ahi = desc_hi(asbo);
+  const uint32_t b0 = desc_lo(b, core * 16u), bk = b0 + core * (uint32_t)(1 + skip);
+  const uint32_t a0 = desc_lo(a, 128);
+  for (int c0 = 0; c0 < 8 * n; c0 += 256)
+    mma_f16(one, tm + c0, desc_lo(bias, 2048), desc_hi(128), b0 + c0, bhi,
+            idesc_f16(min((8 * n - c0 + 15) & ~15, 256), false), 0);
+  for (int i = 0; i < 8; ++i)
+    for (int c0 = 0; c0 < (8 - i) * n; c0 += 256) {
+      const uint32_t id = idesc_f16(min(((8 - i) * n - c0 + 15) & ~15, 256), true);
+      const uint32_t d = tm + (uint32_t)(i * n + c0), al = a0 + (uint32_t)i * (ad >> 4);
+      uint32_t bl = bk + (uint32_t)c0;
+      for (int ks = 0; ks < own; ++ks, bl += 2 * core)
+        mma_f16(one, d, al + 16u * ks, ahi, bl, bhi, id, 1);
+      if (part) {
+        for (int ks = 0; ks < own; ++ks, bl += 2 * core)
+          mma_f16(one, d, al + (part >> 4) + 16u * ks, ahi, bl, bhi, id, 1);
+        if (odd)
+          mma_f16(one, d, (al & 0xFFFFu) + 16u * own + ((part >> 4) << 16), ahi, bl, bhi, id, 1);
+      }
+    }
+}
+
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t one;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xFFFFFFFF;\n selp.u32 %0, 1, 0, p;\n}\n"
+               : "=r"(one));
+  return one;
+}
+
+__device__ __forceinline__ void mma_commit(uint32_t one, uint32_t bar) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n"
+      :: "r"(bar), "r"(one) : "memory");
+}
+
+// Four consecutive tensor-memory columns of this warp's 32 lanes, for each of the
+// eight orders (n columns apart): b[o][e].
+__device__ __forceinline__ void tm_ld(uint32_t addr, int n, uint32_t (&b)[8][4]) {
+#pragma unroll
+  for (int o = 0; o < 8; ++o)
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(b[o][0]), "=r"(b[o][1]), "=r"(b[o][2]), "=r"(b[o][3])
+                 : "r"(addr + (uint32_t)(o * n)));
+}
+// Waits for the loads of b (its registers are operands: no use moves ahead).
+__device__ __forceinline__ void tm_wait(uint32_t (&b)[8][4]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int o = 0; o < 8; ++o)
+    asm volatile("" : "+r"(b[o][0]), "+r"(b[o][1]), "+r"(b[o][2]), "+r"(b[o][3]));
+}
+
+// 64-bit fixed point of v relative to 2^(emax - 1022), 61 bits below it, plus the
+// digit bias; EM = emax << 20 | 0xFFFFF with emax >= 64 (zeros and subnormals then
+// shift out completely).
+__device__ __forceinline__ uint64_t to_fixed(double v, uint32_t EM) {
+  const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+  const uint32_t s = (EM - (hi & 0x7FFFFFFFu)) >> 20;
+  const uint64_t m = ((uint64_t)((hi & 0xFFFFFu) | 0x100000u) << 32 | lo) << 8;
+  uint64_t x;
+  asm("shr.u64 %0, %1, %2;" : "=l"(x) : "l"(m), "r"(s));   // shifts of 64 and more give 0
+  // two's complement and digit bias in one addition
+  const uint32_t sg = (uint32_t)((int32_t)hi >> 31);
+  const uint32_t xl = (uint32_t)x ^ sg, xh = (uint32_t)(x >> 32) ^ sg;
+  return (((uint64_t)xh << 32) | xl) + ((0x80808080ull << 32) | (uint64_t)(0x80808080u - sg));
+}
+
+__device__ __forceinline__ uint64_t mad_wide(uint32_t a, uint32_t b, uint64_t c) {
+  uint64_t r;
+  asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+}
+
+// sum_o b_o 256^(7-o) / 256 without the accumulators' offset, as a signed 64-bit
+// integer (modulo 2^64; the true value stays below 2^62).
+__device__ __forceinline__ int64_t recombine(uint32_t b0, uint32_t b1, uint32_t b2, uint32_t b3,
+                                             uint32_t b4, uint32_t b5, uint32_t b6, uint32_t b7) {
+  constexpr uint64_t M = kMagic;
+  constexpr uint64_t C = 0ull - ((M << 48) + (M << 40) + (M << 32) + (M << 24) + (M << 16) +
+                                 (M << 8) + M + (M >> 8));
+  uint64_t r = mad_wide(b5, 256u, C);
+  r = mad_wide(b4, 65536u, r);
+  r = mad_wide(b3, 16777216u, r);
+  r = mad_wide(b6 + (b7 >> 8), 1u, r);
+  const uint32_t h = b0 * 65536u + (b1 * 256u + b2);
+  return (int64_t)(r + ((uint64_t)h << 32));
+}
+
+// R 2^q as a double, qb = q + 1022: rounded to nearest on the integer units. Rare
+// values (|R| < 2^32, exponents near the ends of the range, NaN blocks) take the
+// careful path.
+__device__ __noinline__ double to_double_slow(int64_t R, int qb) {
+  if (qb > 4000) return __longlong_as_double(0x7FF8000000000000ll);   // the block holds Inf or NaN
+  if (R == 0) return 0.0;
+  return scalbn((double)R, qb - 1022);
+}
+
+// The fast path without its checks, e0 = (q + 1022 + 62) << 20; the result is wrong
+// where |R| < 2^32 (the high word of |R| is returned in `top`).
+__device__ __forceinline__ double to_double_fast(int64_t R, int e0, uint32_t& top) {
+  const int32_t sg = (int32_t)(R >> 63);
+  const uint32_t hi = (uint32_t)((uint64_t)R >> 32) ^ (uint32_t)sg;
+  const uint32_t lo = (uint32_t)R ^ (uint32_t)sg;
+  top = hi;
+  const int sh = __clz((int)hi) - 1;
+  const uint32_t h2 = __funnelshift_l(lo, hi, sh), l2 = lo << (sh & 31);
+  const uint64_t w = (((uint64_t)h2 << 32) | l2) + 0x200u;
+  const uint32_t wh = (uint32_t)(w >> 32), wl = (uint32_t)w;
+  const uint32_t dl = __funnelshift_r(wl, wh, 10);
+  const uint32_t dh = (wh >> 10) + (uint32_t)(e0 - (sh << 20));
+  return __hiloint2double((int)(dh | ((uint32_t)sg & 0x80000000u)), (int)dl);
+}
+
+// The four recombined sums of one thread.
+__device__ __forceinline__ void recombine4(const uint32_t (&b)[8][4], int64_t (&R)[4]) {
+#pragma unroll
+  for (int e = 0; e < 4; ++e)
+    R[e] = recombine(b[0][e], b[1][e], b[2][e], b[3][e], b[4][e], b[5][e], b[6][e], b[7][e]);
+}
+// y[e] = R[e] 2^q[e], qb[e] = q[e] + 1022; one branch for the rare careful cases of all
+// four (lim = 1, or ~0 where the block needs them all).
+__device__ __forceinline__ void to_double4(const int64_t (&R)[4], const int (&qb)[4], uint32_t lim,
+                                           double (&y)[4]) {
+  uint32_t top[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) y[e] = to_double_fast(R[e], (qb[e] + 62) << 20, top[e]);
+  if (min(min(top[0], top[1]), min(top[2], top[3])) < lim) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (top[e] < lim) y[e] = to_double_slow(R[e], qb[e]);
+  }
+}
+// 2^n as a double, -1022 < n < 1023
+__device__ __forceinline__ double pow2(int n) { return __hiloint2double((1023 + n) << 20, 0); }
+__device__ __forceinline__ uint32_t slow_limit(int qb) {
+  return (uint32_t)(qb - 1) > 1900u ? 0xFFFFFFFFu : 1u;
+}
+
+// The fixed-point key of a block: its largest exponent, at least 64, and a mantissa of ones.
+__device__ __forceinline__ uint32_t fixed_key(uint32_t mx) {
+  return ((uint32_t)max((int)(mx >> 20), 64) << 20) | 0xFFFFFu;
+}
+
+// The exponent base of a block: emax of the stored maximum (high word of |v|),
+// 5000 for a block with an infinity or a NaN.
+__device__ __forceinline__ int block_exp(uint32_t mx) {
+  const int e = (int)(mx >> 20);
+  return e == 2047 ? 5000 : max(e, 64);
+}
+
+// Digits of 8 fixed-point values: P[w][h] packs 16-bit pieces of the values, two
+// values per word: P[q][0..3] = bytes (2q, 2q+1) of values (0,1), (2,3), (4,5), (6,7).
+__device__ __forceinline__ void pack_pairs(const uint64_t (&x)[8], int q, uint32_t (&w)[4]) {
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    const uint32_t a = q < 2 ? (uint32_t)x[2 * p] : (uint32_t)(x[2 * p] >> 32);
+    const uint32_t b = q < 2 ? (uint32_t)x[2 * p + 1] : (uint32_t)(x[2 * p + 1] >> 32);
+    w[p] = __byte_perm(a, b, (q & 1) ? 0x7632 : 0x5410);
+  }
+}
+__device__ __forceinline__ uint4 digit_of(const uint32_t (&w)[4], bool high) {
+  const uint32_t s = high ? 0x4341 : 0x4240;
+  return make_uint4(__byte_perm(w[0], 0, s), __byte_perm(w[1], 0, s), __byte_perm(w[2], 0, s),
+                    __byte_perm(w[3], 0, s));
+}
+
+// Bias operand of the first MMA: every row [0.75, 2^-11, 2^-17, 0...].
+__device__ __forceinline__ void fill_bias(unsigned char* ca, int rows) {
+  for (int r = threadIdx.x; r < rows; r += blockDim.x) {
+    reinterpret_cast<uint4*>(ca)[r] = make_uint4(0x10003A00u, 0x00000080u, 0u, 0u);
+    reinterpret_cast<uint4*>(ca)[rows + r] = make_uint4(0u, 0u, 0u, 0u);
+  }
+}
+
+__device__ __forceinline__ void copy_in(unsigned char* dst, const void* src, int bytes) {
+  const uint4* s = reinterpret_cast<const uint4*>(src);
+  for (int x = threadIdx.x; x < bytes / 16; x += blockDim.x) reinterpret_cast<uint4*>(dst)[x] = s[x];
+}
+
+// ============================================================================
+// Two-axis passes. A tile is Na x Nb x 8 points (a, b, x):
+//  * angular: a = Theta, b = Phi, x = eight angular blocks;
+//  * plane: a = theta, b = phi, x = eight Phi columns, four of each half circle.
+// The a axis is a double-Fourier-sphere axis: its operator takes the line and the
+// line of the partner (b + Nb/2; in the plane pass also the column of the other
+// half circle). The b axis is periodic. Both contractions read the tile's digits
+// as MN-major operands, rows (b, x) or (a, x) in groups of 8 x:
+//   copy 1 [digit][b in 0..Nb-1, 0..Nb/2-1][a][8 x]   -- K along a; the partner's
+//           rows start Nb/2 groups further on, hence the repeated first half;
+//   copy 2 [digit][a][b][8 x]                          -- K along b.
+// The Fourier results (and, in the angular pass, the Phi sums that make up the
+// scattering moments) go through shared memory to the threads that finish the
+// points from the DFS results.
+enum EmuPass { EP_ANGULAR = 0, EP_PLANE = 1 };
+
+struct EmuArgs {
+  const double* U;
+  double* K;
+  double sgn;
+  int collision, cons;
+  int vec;   // plane: four columns start on 32 bytes and lie in one half circle
+  long long ntiles;
+};
+
+struct MatArg {
+  const uint16_t* dev;
+  int se;          // 3 - s of the whole matrix
+};
+
+// Adds w, summed over the warp's rows of the same x (lanes 8 apart), to a shared sum.
+__device__ __forceinline__ void moment(unsigned long long* s, int64_t w) {
+  w += __shfl_xor_sync(0xFFFFFFFFu, w, 8);
+  w += __shfl_xor_sync(0xFFFFFFFFu, w, 16);
+  if ((threadIdx.x & 31) < 8) atomicAdd(s, (unsigned long long)w);
+}
+// The shift that makes room for the coefficient sinTh cot th.
+__device__ __forceinline__ int cot_shift(double cot, int delta) {
+  const int e = (int)((uint32_t)__double2hiint(cot) >> 20 & 0x7FFu) - 1023;   // 0: far below
+  return max(1, 2 + delta + e);
+}
+
+__device__ __forceinline__ void cp8(uint32_t dst, const double* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" :: "r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp8_wait() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// Where a tile lies in the field.
+template <int PASS>
+struct TileAt {
+  long long b0 = 0, base = 0;   // angular: first block; plane: (g, i, Theta) offset
+  int k = 0, i = 0, m0 = 0;
+};
+template <int PASS>
+__device__ __forceinline__ TileAt<PASS> tile_at(const Dims& d, long long tile) {
+  TileAt<PASS> r;
+  if (PASS == EP_ANGULAR) {
+    r.b0 = tile * 8;
+  } else {
+    const unsigned nch = (unsigned)(d.NP / 2 + 3) / 4u;
+    unsigned q = (unsigned)tile;   // tiles of a field fit 32 bits (checked on the host)
+    r.m0 = (int)(q % nch) * 4;
+    q /= nch;
+    r.k = (int)(q % (unsigned)d.NT);
+    q /= (unsigned)d.NT;
+    r.i = (int)(q % (unsigned)d.Nr);
+    r.base = (long long)(q / (unsigned)d.Nr) * d.S_g + (long long)r.i * d.S_i +
+             (long long)r.k * d.NP;
+  }
+  return r;
+}
+// The values of this thread's units (zero outside the tile).
+template <int PASS, int U>
+__device__ __forceinline__ void load_units(const Dims& d, const double* F, const TileAt<PASS>& at,
+                                           int S, int hP, int Nb, bool vec, const int (&ua)[U],
+                                           const int (&ub)[U], double (&v)[U][8]) {
+#pragma unroll
+  for (int q = 0; q < U; ++q) {
+#pragma unroll
+    for (int x = 0; x < 8; ++x) v[q][x] = 0.0;
+    if (ua[q] < 0) continue;
+    if (PASS == EP_ANGULAR) {
+      const double* src = F + at.b0 * S + ua[q] * Nb + ub[q];
+#pragma unroll
+      for (int x = 0; x < 8; ++x)
+        if (at.b0 + x < d.nblk) v[q][x] = src[x * S];
+    } else {
+      const double* src = F + at.base + (long long)ua[q] * d.S_j + (long long)ub[q] * d.S_l + at.m0;
+      if (vec) {   // four columns of a half circle at once: every lane reads its own line
+#pragma unroll
+        for (int x = 0; x < 8; x += 4)
+          asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
+                       : "=d"(v[q][x]), "=d"(v[q][x + 1]), "=d"(v[q][x + 2]), "=d"(v[q][x + 3])
+                       : "l"(src + (x ? hP : 0)));
+      } else {
+#pragma unroll
+        for (int x = 0; x < 8; ++x)
+          if (at.m0 + (x & 3) < hP) v[q][x] = src[(x & 3) + (x >= 4 ? hP : 0)];
+      }
+    }
+  }
+}
+
+// NA_, NB_: the axes' lengths at compile time (0: from the geometry).
+template <int PASS, int KF, int T, int U, int NA_, int NB_>
+__global__ void __launch_bounds__(T, T == 256 ? 2 : 1)
+k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
+  extern __shared__ __align__(128) unsigned char sm[];
+  const Dims& d = p.d;
+  const uint32_t smb = sm_u32(sm);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int uwarp = __shfl_sync(0xFFFFFFFFu, warp, 0);   // warp-uniform
+  constexpr int NG = T / 128;                     // threads per tensor-memory lane
+  const int Na = NA_ ? NA_ : g.Na, Nb = NB_ ? NB_ : g.Nb, hb = Nb / 2, exP = Na * 8 + 8;
+  // small arrays
+  unsigned char* ms = sm + g.oMs;
+  uint64_t* bar = reinterpret_cast<uint64_t*>(ms);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(ms + 16);
+  volatile int* dead = reinterpret_cast<volatile int*>(ms + 20);  // a wait ran out
+  uint32_t* smax = reinterpret_cast<uint32_t*>(ms + 32);          // [2][8]
+  double* xs = reinterpret_cast<double*>(ms + 96);                // [2][8][8] scalars of a tile's x
+  double* xm = xs + 2 * 64;                                       // [10][8] moments
+  unsigned long long* jsum = reinterpret_cast<unsigned long long*>(xm + 80);   // [10][8]
+  int64_t* wqt = reinterpret_cast<int64_t*>(jsum + 80);           // angular: weights [Na]
+  int* hs = reinterpret_cast<int*>(jsum + 80);                    // plane: shifts [Na]
+  int64_t* ex = reinterpret_cast<int64_t*>(sm + g.oEx);           // [Nb][a][8 x]
+
+  if (Na % 8 || Nb % 16) {   // K paddings read as zero
+    for (int x = tid; x < g.oB1 / 16; x += T)
+      reinterpret_cast<uint4*>(sm)[x] = make_uint4(0, 0, 0, 0);
+  }
+  if (tid < 16) smax[tid] = 0;
+  if (tid == 0) *dead = 0;
+  copy_in(sm + g.oB1, m1.dev, (1 + g.kc1) * g.r1 * 16);
+  copy_in(sm + g.oB2, m2.dev, (1 + g.kc2) * g.r2 * 16);
+  fill_bias(sm + g.oCA, 128);
+  if (tid == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(sm_u32(&bar[0])) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(sm_u32(&bar[1])) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                 :: "r"(sm_u32(tslot)), "r"(g.cols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, *tslot, 0);
+
+  // this thread's (a, b) units: all eight x of each
+  int ua[U], ub[U];
+#pragma unroll
+  for (int q = 0; q < U; ++q) {
+    const int u = tid + q * T;
+    ua[q] = u < Na * Nb ? u / Nb : -1;
+    ub[q] = u - (u / Nb) * Nb;
+  }
+  const int row = (warp & 3) * 32 + lane, grp = warp >> 2, rx = row & 7, rg = row >> 3;
+  const int jobs = g.mt2 + g.mt1, ahead = g.dual ? 2 : 1;
+  const int S = PASS == EP_ANGULAR ? Na * Nb : d.NT * d.NP, hP = d.NP / 2;
+  // The combination W of the two contractions stays in fixed point: a multiply of two
+  // 64-bit integers costs about a sixth of an FP64 one here. Unit of W: 2^h times that
+  // of the DFS results; h makes room for the Fourier term's coefficient, delta is the
+  // difference of the two matrices' scales.
+  const int delta = m2.se - m1.se;
+  for (int a = tid; a < Na; a += T) {
+    if (PASS == EP_PLANE)
+      hs[a] = max(2, 3 + delta + ilogb(t.inv_sinth[a]));
+    else   // weights of the moments (Fejer x trapezoid; conservative: of Fhat / sinTh)
+      wqt[a] = __double2ll_rn((A.cons ? t.qdir[a] / t.sinT[a] : t.qdir[a]) * pow2(63));
+  }
+  double v[U][8];
+  TileAt<PASS> at{};
+  // block z of tile `at`: the epilogue's constants, as asynchronous copies (their
+  // latency is nobody's): 1/r, kappa, cot th, eta, kappa_s, kappa_s' b, c, sin th
+  auto scalars_load = [&](int z, int bf) {
+    const long long blk = at.b0 + z < d.nblk ? at.b0 + z : 0;
+    const unsigned q = (unsigned)blk / (unsigned)d.Np;
+    const unsigned jj = q % (unsigned)d.Nt, ii = q / (unsigned)d.Nt % (unsigned)d.Nr;
+    const uint32_t x = sm_u32(xs + bf * 64 + z);
+    cp8(x, t.inv_r + ii);
+    cp8(x + 64, p.kap + blk);
+    cp8(x + 128, t.cot_th + jj);
+    cp8(x + 192, p.eta + blk);
+    cp8(x + 256, p.kaps + blk);
+    if (KF >= KF_LINEAR && p.scb) cp8(x + 320, p.scb + blk);
+    if (KF >= KF_QUADRATIC) cp8(x + 384, p.scc + blk);
+    cp8(x + 448, t.sin_th + jj);
+  };
+  if ((long long)blockIdx.x < A.ntiles) {
+    at = tile_at<PASS>(d, blockIdx.x);
+    load_units<PASS, U>(d, A.U, at, S, hP, Nb, A.vec, ua, ub, v);
+    if (PASS == EP_ANGULAR && warp == 1 && lane < 8) scalars_load(lane, 0);
+  }
+  int coef_n = -1;   // the Fourier coefficient this thread holds, and for what
+  double coef_key = 0.0;
+  int64_t coef = 0, ws = 0, wc = 0;
+  int cth_b = -1;    // plane: cosPh of its DFS rows, and of which
+  int64_t cth = 0;
+  uint32_t phase = 0;   // one bit per barrier
+  bool alive = true;
+  int buf = 0;
+  for (long long tile = blockIdx.x; tile < A.ntiles && alive; tile += gridDim.x, buf ^= 1) {
+    // ---- largest magnitude of each block (angular) or of the tile (plane)
+    {
+      uint32_t mx[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+#pragma unroll
+      for (int q = 0; q < U; ++q)
+#pragma unroll
+        for (int x = 0; x < 8; ++x)
+          mx[x] = max(mx[x], (uint32_t)__double2hiint(v[q][x]) & 0x7FFFFFFFu);
+      if (PASS == EP_PLANE) {
+#pragma unroll
+        for (int x = 1; x < 8; ++x) mx[0] = max(mx[0], mx[x]);
+        const uint32_t r = __reduce_max_sync(0xFFFFFFFFu, mx[0]);
+        if (lane == 0) atomicMax(&smax[buf * 8], r);
+      } else {
+        uint32_t mine = 0;
+#pragma unroll
+        for (int x = 0; x < 8; ++x) {
+          const uint32_t r = __reduce_max_sync(0xFFFFFFFFu, mx[x]);
+          if (lane == x) mine = r;
+        }
+        if (lane < 8) atomicMax(&smax[buf * 8 + lane], mine);
+      }
+    }
+    if (PASS == EP_ANGULAR && warp == 1) cp8_wait();   // this tile's scalars
+    __syncthreads();   // the maxima and scalars; the previous tile is finished
+    if (tid < 8) smax[(buf ^ 1) * 8 + tid] = 0;
+    if (PASS == EP_ANGULAR && tid < 80) jsum[tid] = 0;
+    // ---- digits
+    {
+      uint32_t em[8];
+#pragma unroll
+      for (int x = 0; x < 8; ++x)
+        em[x] = fixed_key(smax[buf * 8 + (PASS == EP_PLANE ? 0 : x)]);
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        if (ua[q] < 0) continue;
+        uint64_t f[8];
+#pragma unroll
+        for (int x = 0; x < 8; ++x) f[x] = to_fixed(v[q][x], em[x]);
+        unsigned char* c1 = sm + g.oC1 + ub[q] * g.sb1 + ua[q] * 16;
+        unsigned char* c2 = sm + g.oC2 + ua[q] * g.sb2 + ub[q] * 16;
+        const bool ring = ub[q] < hb, rot = PASS == EP_PLANE && !ring;
+#pragma unroll
+        for (int w = 3; w >= 0; --w) {
+          uint32_t pk[4];
+          pack_pairs(f, w, pk);
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int dig = 7 - (2 * w + h);
+            const uint4 x4 = digit_of(pk, h);
+            *reinterpret_cast<uint4*>(c2 + dig * g.d2) = x4;
+            const uint4 y4 = rot ? make_uint4(x4.z, x4.w, x4.x, x4.y) : x4;
+            *reinterpret_cast<uint4*>(c1 + dig * g.d1) = y4;
+            if (ring) *reinterpret_cast<uint4*>(c1 + dig * g.d1 + Nb * g.sb1) = y4;
+          }
+        }
+      }
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    // issues job n (one call site: the unrolled chains are inlined there, their
+    // operands in uniform registers)
+    auto issue = [&](int n) {
+      const uint32_t r = g.dual ? (uint32_t)(n & 1) : 0u;
+      const uint32_t one = elect_one(), tm = tmem + r * (uint32_t)g.half, ca = smb + g.oCA;
+      if (n < g.mt2) {
+        const uint32_t a = smb + g.oC2 + (uint32_t)(16 * n * g.sb2), b = smb + g.oB2;
+        if ((NB_ ? NB_ <= 16 : g.kc2 == 2) && g.n2 <= 32)
+          chain_steps<1, false, false>(one, tm, ca, a, g.d2, g.sb2, 0, b, 0, g.r2, g.n2);
+        else if (!NB_ && g.kc2 == 4 && g.n2 <= 32)
+          chain_steps<2, false, false>(one, tm, ca, a, g.d2, g.sb2, 0, b, 0, g.r2, g.n2);
+        else
+          chain_any(one, tm, ca, a, g.d2, g.sb2, g.kc2 / 2, 0, false, b, 0, g.r2, g.n2);
+      } else {
+        const uint32_t a = smb + g.oC1 + (uint32_t)(16 * (n - g.mt2) * g.sb1), b = smb + g.oB1;
+        const uint32_t part = (uint32_t)(hb * g.sb1);
+        const int ka = NA_ ? (NA_ + 7) / 8 : g.n1 <= 32 ? g.ka : 0;
+        if (ka == 1)
+          chain_steps<0, true, true>(one, tm, ca, a, g.d1, g.sb1, part, b, 0, g.r1, g.n1);
+        else if (ka == 2)
+          chain_steps<1, true, false>(one, tm, ca, a, g.d1, g.sb1, part, b, 0, g.r1, g.n1);
+        else if (ka == 3)
+          chain_steps<1, true, true>(one, tm, ca, a, g.d1, g.sb1, part, b, 0, g.r1, g.n1);
+        else if (ka == 4)
+          chain_steps<2, true, false>(one, tm, ca, a, g.d1, g.sb1, part, b, 0, g.r1, g.n1);
+        else
+          chain_any(one, tm, ca, a, g.d1, g.sb1, g.ka / 2, part, g.ka & 1, b, 0, g.r1, g.n1);
+      }
+      mma_commit(one, sm_u32(&bar[r]));
+      __syncwarp();
+    };
+    const TileAt<PASS> cur = at;
+    int issued = 0;
+    // waits for job n, every warp for itself; where a wait runs out the warp goes on (its
+    // results are void) and all leave together after the job's barrier
+    auto wait_job = [&](int n) {
+      const uint32_t r = g.dual ? (uint32_t)(n & 1) : 0u;
+      if (!bar_wait(sm_u32(&bar[r]), (phase >> r) & 1u, p.wait_operand)) *dead = 1;
+      phase ^= 1u << r;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    };
+    auto end_job = [&](int n) {
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncthreads();
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      if (*dead) {
+        if (tid == 0 && p.err) atomicExch(p.err, 1);
+        // our own MMAs end before the CTA exits (full bound)
+        for (int x = n; x < issued; ++x) {
+          const uint32_t rr = g.dual ? (uint32_t)(x & 1) : 0u;
+          bar_wait(sm_u32(&bar[rr]), ((phase >> rr) & 1u) ^ (x == n ? 1u : 0u), kDefaultWaitIters);
+        }
+        return false;
+      }
+      return true;
+    };
+    auto lanes = [&](int n) {   // this warp's tensor-memory address in job n's region
+      const uint32_t r = g.dual ? (uint32_t)(n & 1) : 0u;
+      return tmem + r * (uint32_t)g.half + ((uint32_t)((warp & 3) * 32) << 16);
+    };
+    const int eb = block_exp(smax[buf * 8 + (PASS == EP_PLANE ? 0 : rx)]);
+    const double* xc = xs + buf * 64;   // the scalars of this tile
+    for (int n = 0; n < jobs; ++n) {
+      for (const int upto = min(n + ahead, jobs); issued < upto; ++issued)
+        if (uwarp == T / 32 - 1) issue(issued);
+      if (n == 0) {
+        // the next tile's values travel while this one is finished
+        if (tile + gridDim.x < A.ntiles) {
+          at = tile_at<PASS>(d, tile + gridDim.x);
+          load_units<PASS, U>(d, A.U, at, S, hP, Nb, A.vec, ua, ub, v);
+          if (PASS == EP_ANGULAR && warp == 1 && lane < 8) scalars_load(lane, buf ^ 1);
+        }
+      }
+      if (n < g.mt2) {
+      // ---- Fourier results: rows (a, x), times the coefficient of their term
+      const int a = 16 * n + rg;
+      const bool val = a < Na;
+      // the row's coefficient: sinTh cot th (angular), sinPh / sin th (plane). The
+      // CTA's next tile mostly has the same th or Phi columns: kept while it does
+      const double key = PASS == EP_ANGULAR ? xc[16 + rx] : (double)cur.m0;
+      if (n != coef_n || key != coef_key) {
+        coef_n = n;
+        coef_key = key;
+        coef = ws = wc = 0;
+        if (val) {
+          if (PASS == EP_ANGULAR) {
+            const double st = t.sinT[a], ct = t.cosT[a];
+            coef = __double2ll_rn(st * key * pow2(64 + delta - cot_shift(key, delta)));
+            if (KF >= KF_LINEAR) {
+              ws = __double2ll_rn(st * pow2(62));
+              wc = __double2ll_rn(ct * pow2(62));
+            }
+          } else {
+            const bool ok = cur.m0 + (rx & 3) < hP;
+            const double sp = ok ? t.sinP[cur.m0 + (rx & 3) + (rx >= 4 ? hP : 0)] : 0.0;
+            coef = __double2ll_rn(sp * t.inv_sinth[a] * pow2(64 + delta - hs[a]));
+          }
+        }
+      }
+      wait_job(n);
+      const uint32_t tl = lanes(n);
+      const int nreal = Nb + (PASS == EP_ANGULAR && A.collision ? g.nf - g.nz : 0);
+      int64_t* exr = ex + a * 8 + rx;
+      for (int q = grp; 4 * q < nreal; q += NG) {
+        uint32_t bb[8][4];
+        tm_ld(tl + (uint32_t)(4 * q), g.n2, bb);
+        tm_wait(bb);
+        int64_t R[4];
+        recombine4(bb, R);
+        // functionals: outputs 0 and Nb/2 (whose derivative rows vanish, nz of them) and
+        // those from Nb on
+        const bool special = PASS == EP_ANGULAR &&
+                             ((g.nz > 0 && q == 0) || (g.nz > 1 && q == hb / 4) || 4 * q + 4 > Nb);
+        if (!special) {
+          if (val) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              if (4 * q + e < Nb) exr[(4 * q + e) * exP] = __mul64hi(R[e], coef);
+          }
+          continue;
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int o = 4 * q + e;
+          if (o >= nreal) break;
+          const bool zero = g.nz > 0 && (o == 0 || (g.nz > 1 && o == hb));
+          if (o < Nb && val) exr[o * exP] = zero ? 0 : __mul64hi(R[e], coef);
+          const int f = o >= Nb ? o - Nb + g.nz : !zero ? -1 : o == 0 ? 0 : 1;
+          if (f < 0 || !A.collision) continue;
+          // Phi sums of F times {1, cos, sin, cos^2, cos sin}: their Theta sums are the
+          // scattering moments, summed as integers (exact, in any order). Unit: 2 of R's
+          // for the weight alone, times 4 for every further factor
+          const int64_t w1 = val ? __mul64hi(R[e], wqt[a]) : 0;
+          if (f == 0) {
+            moment(jsum + rx, w1);
+            if (KF >= KF_LINEAR) moment(jsum + 8 + rx, __mul64hi(w1, wc));
+            if (KF >= KF_QUADRATIC) moment(jsum + 32 + rx, __mul64hi(__mul64hi(w1, wc), wc));
+          } else if (f < 3) {
+            const int64_t w2 = __mul64hi(w1, ws);
+            moment(jsum + 8 * (1 + f) + rx, w2);
+            if (KF >= KF_QUADRATIC) moment(jsum + 8 * (6 + f) + rx, __mul64hi(w2, wc));
+          } else {
+            moment(jsum + 8 * (2 + f) + rx, __mul64hi(__mul64hi(w1, ws), ws));
+          }
+        }
+      }
+      } else {
+      // ---- DFS results: rows (b, x); every point is finished here
+      const int b = 16 * (n - g.mt2) + rg;
+      const int w = PASS == EP_PLANE && b >= hb ? rx ^ 4 : rx;
+      bool val = b < Nb;
+      double* Kp;
+      const double* Ip;   // what the epilogue reads per point: U (angular) or K (plane)
+      unsigned st;        // stride of a (a plane spans less than 2^32 elements)
+      if (PASS == EP_ANGULAR) {
+        val = val && cur.b0 + rx < d.nblk;
+        const long long o = (cur.b0 + rx) * S + b;
+        Kp = A.K + o;
+        Ip = A.U + o;
+        st = Nb;
+      } else {
+        val = val && cur.m0 + (w & 3) < hP;
+        Kp = A.K + cur.base + (long long)b * d.S_l + cur.m0 + (w & 3) + (w >= 4 ? hP : 0);
+        Ip = Kp;
+        st = (unsigned)d.S_j;
+      }
+      const bool rd = val && (PASS == EP_PLANE || A.collision);
+      double in[2][4];
+      auto load_in = [&](int q) {   // quads q and q + NG
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int a = 4 * (q + h * NG) + e;
+            in[h][e] = rd && a < Na ? Ip[(unsigned)a * st] : 0.0;
+          }
+      };
+      load_in(grp);
+      wait_job(n);
+      const uint32_t tl = lanes(n);
+      double c0, kks = 0.0, src = 0.0, hr = 0.0, hc = 0.0, mrr = 0.0, qmc = 0.0, rmc = 0.0;
+      int hx = 0;
+      if (PASS == EP_PLANE) {
+        c0 = A.sgn * t.sinT[cur.k] * t.inv_r[cur.i];
+        if (cth_b != b * 64 + cur.m0) {   // cosPh as a fixed-point coefficient of the DFS term
+          cth_b = b * 64 + cur.m0;
+          cth = val ? __double2ll_rn(t.cosP[cur.m0 + (w & 3) + (w >= 4 ? hP : 0)] * pow2(62)) : 0;
+        }
+      } else {
+        c0 = -A.sgn * xc[w];
+        hx = cot_shift(xc[16 + w], delta);
+        if (A.collision) {
+          const double ks = xc[32 + w], J = xm[w];
+          kks = xc[8 + w] + ks;
+          src = fma(ks, J, A.cons ? xm[72 + w] : xc[24 + w]);
+          if (KF >= KF_LINEAR) {
+            const double cp = t.cosP[val ? b : 0], sp = t.sinP[val ? b : 0];
+            const double kb = p.scb ? ks * xc[40 + w] : 0.0;
+            hr = kb * xm[8 + w];
+            hc = kb * (cp * xm[16 + w] + sp * xm[24 + w]);
+            if (KF >= KF_QUADRATIC) {
+              // M_phph = J - M_rr - M_thth (the trace of omega omega is 1)
+              const double kc = ks * xc[48 + w], j3 = J * (1.0 / 3.0);
+              const double rr = xm[32 + w], tt = xm[40 + w];
+              mrr = kc * (rr - j3);
+              qmc = kc * (cp * cp * (tt - j3) + sp * sp * (J - rr - tt - j3) +
+                          2.0 * cp * sp * xm[48 + w]);
+              rmc = 2.0 * kc * (cp * xm[56 + w] + sp * xm[64 + w]);
+            }
+          }
+        }
+      }
+      const int qv = eb + m1.se;
+      const uint32_t lim = slow_limit(qv);
+      const int64_t* exr = ex + (val ? b : 0) * exP + w;
+      for (int q0 = grp; 4 * q0 < Na; q0 += 2 * NG) {
+        if (q0 != grp) load_in(q0);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int q = q0 + h * NG;
+          if (4 * q >= Na) break;
+          uint32_t bb[8][4];
+          tm_ld(tl + (uint32_t)(4 * q), g.n1, bb);
+          tm_wait(bb);
+          int64_t W[4];
+          int qb[4];
+          recombine4(bb, W);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int a = min(4 * q + e, Na - 1);
+            const int ha = PASS == EP_ANGULAR ? hx : hs[a];
+            if (PASS == EP_ANGULAR) W[e] >>= hx;
+            else W[e] = __mul64hi(W[e], cth) >> (ha - 2);
+            W[e] += exr[a * 8];
+            qb[e] = qv + ha;
+          }
+          double y4[4];
+          to_double4(W, qb, lim, y4);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int a = 4 * q + e;
+            if (a >= Na) break;
+            double r2;
+            if (PASS == EP_PLANE) {
+              r2 = fma(c0, y4[e], in[h][e]);
+            } else {
+              double col = 0.0;
+              if (A.collision) {
+                double gain = src;
+                if (KF >= KF_LINEAR) {
+                  const double ct = t.cosT[a], sT = t.sinT[a];
+                  double u1 = hr, u2 = hc;
+                  if (KF >= KF_QUADRATIC) {
+                    u1 = fma(ct, mrr, fma(sT, rmc, hr));
+                    u2 = fma(sT, qmc, hc);
+                  }
+                  gain = fma(ct, u1, fma(sT, u2, gain));
+                }
+                if (A.cons) gain *= t.sinT[a];
+                col = fma(-kks, in[h][e], gain);
+              }
+              r2 = fma(c0, y4[e], col);
+            }
+            if (val) Kp[(unsigned)a * st] = r2;
+          }
+        }
+      }
+      }
+      alive = end_job(n);
+      if (!alive) break;
+      if (PASS == EP_ANGULAR && n == g.mt2 - 1 && A.collision) {
+        if (tid < 80) {
+      // moment z of block x as a double (visible after the next wait's barrier)
+      const int z = tid >> 3, x = tid & 7;
+      constexpr int nm = KF == KF_ISO ? 1 : KF == KF_LINEAR ? 4 : 9;
+      if (z < nm) {
+        const int more = z == 0 ? 1 : z < 4 ? 3 : 5;   // 2 and 4 per factor, as exponents
+        const int qv = block_exp(smax[buf * 8 + x]) + m2.se + more;
+        uint32_t top;
+        const int64_t R = (int64_t)jsum[tid];
+        double y = to_double_fast(R, (qv + 62) << 20, top);
+        if (top < slow_limit(qv)) y = to_double_slow(R, qv);
+        xm[tid] = y;
+      } else if (z == 9 && A.cons) {   // eta r^2 sin th
+        xm[tid] = xc[24 + x] * xc[56 + x] / (xc[x] * xc[x]);
+      }
+    }
+        __syncthreads();
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;"
+                 :: "r"(tmem), "r"(g.cols) : "memory");
+  }
+}
+
+// ============================================================================
+// Radial pass: 128 (Theta, Phi) columns of one (g, theta, phi) per tile, all N_r
+// nodes. Digits [digit][column / 8][node][8 columns], MN-major; the matrix rows
+// are ordered 0, N, 1, 2, ..., N-1 so that the two Tau rows come first.
+struct RadArgs {
+  const double *U, *Kin;
+  double sgn;
+  int tau, mode;
+  double *F, *Acc, *Uout, *out;
+  double dt;
+  long long ntiles;
+};
+struct RadMats {
+  const uint16_t* dev[8];
+  const int* se[8];
+};
+
+__device__ __forceinline__ void prefetch_line(const double* p) {
+  asm volatile("prefetch.global.L2 [%0];" :: "l"(p));
+}
+
+__device__ __forceinline__ int rad_row(int o, int N) { return o == 0 ? 0 : o == 1 ? N : o - 1; }
+
+template <int T, int MODE>
+__global__ void __launch_bounds__(T, T == 256 ? 2 : 1)
+k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
+  extern __shared__ __align__(128) unsigned char sm[];
+  const Dims& d = p.d;
+  const uint32_t smb = sm_u32(sm);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int uwarp = __shfl_sync(0xFFFFFFFFu, warp, 0);   // warp-uniform
+  constexpr int NG = T / 128;
+  const int Nr = g.Nr, N = Nr - 1, NP = d.NP, S = d.NT * d.NP;
+  unsigned char* ms = sm + g.oMs;
+  uint64_t* bar = reinterpret_cast<uint64_t*>(ms);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(ms + 16);
+  volatile int* dead = reinterpret_cast<volatile int*>(ms + 20);   // a wait ran out
+  uint32_t* smax = reinterpret_cast<uint32_t*>(ms + 24);   // [2]
+  int* se = reinterpret_cast<int*>(ms + 32);               // [ng * n]
+  if (!g.left || Nr != 8 * g.kc + 1) {   // K paddings read as zero
+    for (int x = tid; x < g.oB / 16; x += T)
+      reinterpret_cast<uint4*>(sm)[x] = make_uint4(0, 0, 0, 0);
+  }
+  if (tid < 2) smax[tid] = 0;
+  if (tid == 0) *dead = 0;
+  for (int q = 0; q < g.ng; ++q) {
+    copy_in(sm + g.oB + q * g.bB, M.dev[q], g.bB);
+    for (int x = tid; x < g.n; x += T) se[q * g.n + x] = M.se[q][x];
+  }
+  fill_bias(sm + g.oCA, 128);
+  if (tid == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(sm_u32(&bar[0])) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(sm_u32(&bar[1])) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                 :: "r"(sm_u32(tslot)), "r"(g.cols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, *tslot, 0);
+  const int nch = (S + 127) / 128;
+  const int row = (warp & 3) * 32 + lane, grp = warp >> 2;
+  const int ahead = g.dual ? 2 : 1;
+  // MODE: the update; RAD_STAGE1 stands for stages 1 and 2 (A.mode tells them apart)
+  constexpr bool rA = MODE == RAD_STAGE1 || MODE == RAD_STAGE3 || MODE == RAD_AB2;
+  uint32_t phase = 0;
+  bool alive = true;
+  int buf = 0;
+  constexpr int U = 3;   // (node, 8 columns) units held per thread and round
+  auto coords = [&](long long tile, int& c0, long long& base) {
+    unsigned q0 = (unsigned)tile;   // tiles of a field fit 32 bits (checked on the host)
+    c0 = (int)(q0 % (unsigned)nch) * 128;
+    q0 /= (unsigned)nch;
+    const int l = (int)(q0 % (unsigned)d.Np);
+    q0 /= (unsigned)d.Np;
+    const int j = (int)(q0 % (unsigned)d.Nt);
+    base = (long long)(q0 / (unsigned)d.Nt) * d.S_g + (long long)j * d.S_j +
+           (long long)l * d.S_l + c0;
+  };
+  for (long long tile = blockIdx.x; tile < A.ntiles && alive; tile += gridDim.x, buf ^= 1) {
+    int c0;
+    long long base;
+    coords(tile, c0, base);
+    const int Wc = min(128, S - c0);
+    // the lines the epilogue reads are requested into L2 meanwhile (one 128-byte line
+    // per request)
+    for (int u = tid; u < Nr * 8; u += T) {
+      const int w = (u & 7) * 16;
+      if (w < Wc) {
+        const long long gi = base + (long long)(u >> 3) * d.S_i + w;
+        prefetch_line(A.Kin + gi);
+        if (MODE != RAD_RHS) prefetch_line(A.F + gi);
+        if (rA) prefetch_line(A.Acc + gi);
+      }
+    }
+    // the tile's values, and their largest magnitude; U units a thread are kept in
+    // registers (longer lines are read again for the conversion)
+    double v[U][8];
+    uint32_t mx = 0;
+    auto load_unit = [&](int u, double (&z)[8]) {
+      const int w = (u & 15) * 8;
+#pragma unroll
+      for (int x = 0; x < 8; ++x) z[x] = 0.0;
+      if (u < Nr * 16) {
+        const double* src = A.U + base + (long long)(u >> 4) * d.S_i + w;
+        if (w + 8 <= Wc) {
+#pragma unroll
+          for (int x = 0; x < 8; x += 2) {
+            const double2 y = *reinterpret_cast<const double2*>(src + x);
+            z[x] = y.x;
+            z[x + 1] = y.y;
+          }
+        } else {
+#pragma unroll
+          for (int x = 0; x < 8; ++x)
+            if (w + x < Wc) z[x] = src[x];
+        }
+      }
+    };
+#pragma unroll
+    for (int q = 0; q < U; ++q) load_unit(tid + q * T, v[q]);
+#pragma unroll
+    for (int q = 0; q < U; ++q)
+#pragma unroll
+      for (int x = 0; x < 8; ++x)
+        mx = max(mx, (uint32_t)__double2hiint(v[q][x]) & 0x7FFFFFFFu);
+    for (int u = tid + U * T; u < Nr * 16; u += T) {
+      double z[8];
+      load_unit(u, z);
+#pragma unroll
+      for (int x = 0; x < 8; ++x) mx = max(mx, (uint32_t)__double2hiint(z[x]) & 0x7FFFFFFFu);
+    }
+    mx = __reduce_max_sync(0xFFFFFFFFu, mx);
+    if (lane == 0) atomicMax(&smax[buf], mx);
+    __syncthreads();
+    if (tid == 0) smax[buf ^ 1] = 0;
+    const uint32_t tmax = smax[buf], EM = fixed_key(tmax);
+    const int eb = block_exp(tmax);
+    for (int u0 = tid; u0 < Nr * 16; u0 += U * T) {
+      if (u0 != tid) {
+#pragma unroll
+        for (int q = 0; q < U; ++q) load_unit(u0 + q * T, v[q]);
+      }
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        const int u = u0 + q * T;
+        if (u >= Nr * 16) continue;
+        const int ii = u >> 4, wg = u & 15;
+        uint64_t f[8];
+#pragma unroll
+        for (int x = 0; x < 8; ++x) f[x] = to_fixed(v[q][x], EM);
+        if (g.left && ii == N) {
+          // the leftover node: its eight digits beside the bias, one 16-byte row per column
+#pragma unroll
+          for (int x = 0; x < 8; ++x) {
+            const uint32_t lo = (uint32_t)f[x], hi = (uint32_t)(f[x] >> 32);
+            *reinterpret_cast<uint4*>(sm + g.oCA + 2048 + (wg * 8 + x) * 16) =
+                make_uint4(__byte_perm(hi, 0, 0x4243), __byte_perm(hi, 0, 0x4041),
+                           __byte_perm(lo, 0, 0x4243), __byte_perm(lo, 0, 0x4041));
+          }
+          continue;
+        }
+        unsigned char* c = sm + g.oA + wg * g.sb + ii * 16;
+#pragma unroll
+        for (int w = 3; w >= 0; --w) {
+          uint32_t pk[4];
+          pack_pairs(f, w, pk);
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            *reinterpret_cast<uint4*>(c + (7 - (2 * w + h)) * g.d) = digit_of(pk, h);
+        }
+      }
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    auto issue = [&](int n) {
+      const uint32_t r = g.dual ? (uint32_t)(n & 1) : 0u;
+      const uint32_t one = elect_one(), tm = tmem + r * (uint32_t)g.half;
+      const uint32_t ca = smb + g.oCA, a = smb + g.oA, b = smb + g.oB + (uint32_t)(n * g.bB);
+      if (g.kc == 4)
+        chain_steps<2, false, false>(one, tm, ca, a, g.d, g.sb, 0, b, g.left, g.rows, g.n);
+      else if (g.kc == 2)
+        chain_steps<1, false, false>(one, tm, ca, a, g.d, g.sb, 0, b, g.left, g.rows, g.n);
+      else if (g.kc == 6)
+        chain_steps<3, false, false>(one, tm, ca, a, g.d, g.sb, 0, b, g.left, g.rows, g.n);
+      else if (g.kc == 8)
+        chain_steps<4, false, false>(one, tm, ca, a, g.d, g.sb, 0, b, g.left, g.rows, g.n);
+      else
+        chain_any(one, tm, ca, a, g.d, g.sb, g.kc / 2, 0, false, b, g.left, g.rows, g.n);
+      mma_commit(one, sm_u32(&bar[r]));
+      __syncwarp();
+    };
+    int issued = 0;
+    const bool val = row < Wc;
+    const int kT = val ? (c0 + row) / NP : 0;
+    const double cT = t.cosT[kT], ck = A.sgn * cT;
+    const int bn = cT > 0.0 ? 0 : N;   // inflow node
+    const double* Kc = A.Kin + base + row;
+    const double* Fc = A.F + base + row;
+    const double* Ac = A.Acc + base + row;
+    const unsigned Si = (unsigned)d.S_i;   // a group spans less than 2^32 elements (host)
+    double kb = val && A.tau ? Kc[(unsigned)bn * Si] : 0.0;
+    double* dst = (MODE == RAD_RHS ? A.out
+                   : MODE == RAD_STAGE3 || MODE == RAD_AB2 || MODE == RAD_AB2_START ? A.F
+                                                                                    : A.Uout) +
+                  base + row;
+    double* Aw = A.Acc + base + row;
+    const double cu = MODE == RAD_STAGE3 ? A.dt / 6.0
+                      : MODE == RAD_STAGE0 || (MODE == RAD_STAGE1 && A.mode == RAD_STAGE1)
+                          ? 0.5 * A.dt
+                          : A.dt;
+    double nk[4], nf[4], na[4];
+    unsigned noff[4];
+    auto load_rows = [&](int n, int q, int no) {   // quad q of group n
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int o = 4 * q + e;
+        noff[e] = (unsigned)(o < no ? rad_row(n * g.go + o, N) : 0) * Si;
+        nk[e] = nf[e] = na[e] = 0.0;
+        if (val && o < no) {
+          nk[e] = Kc[noff[e]];
+          if (MODE != RAD_RHS) nf[e] = Fc[noff[e]];
+          if (rA) na[e] = Ac[noff[e]];
+        }
+      }
+    };
+    if (tile + gridDim.x < A.ntiles) {   // the next tile's lines, into L2
+      int c1;
+      long long b1;
+      coords(tile + gridDim.x, c1, b1);
+      for (int u = tid; u < Nr * 8; u += T)
+        if (c1 + (u & 7) * 16 < S)
+          prefetch_line(A.U + b1 + (long long)(u >> 3) * d.S_i + (u & 7) * 16);
+    }
+    for (int n = 0; n < g.ng; ++n) {
+      for (const int upto = min(n + ahead, g.ng); issued < upto; ++issued)
+        if (uwarp == T / 32 - 1) issue(issued);
+      const uint32_t r = g.dual ? (uint32_t)(n & 1) : 0u;
+      const int no = min(g.go, Nr - n * g.go);
+      if (4 * grp < no) load_rows(n, grp, no);
+      // where a wait runs out the warp goes on (its results are void) and all leave
+      // together after the group's barrier
+      if (!bar_wait(sm_u32(&bar[r]), (phase >> r) & 1u, p.wait_operand)) *dead = 1;
+      phase ^= 1u << r;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t tl = tmem + r * (uint32_t)g.half + ((uint32_t)((warp & 3) * 32) << 16);
+      if (n == 0 && A.tau) {   // the finished rate at the inflow node (both rows lead this group)
+        uint32_t b[8][4];
+        tm_ld(tl, g.n, b);
+        tm_wait(b);
+        const int qb[4] = {eb + se[0], eb + se[1], 0, 0};
+        int64_t R[4];
+        recombine4(b, R);
+        double y4[4];
+        to_double4(R, qb, max(slow_limit(qb[0]), slow_limit(qb[1])), y4);
+        kb = fma(ck, bn == 0 ? y4[0] : y4[1], kb);
+        if ((N - bn) & 1) kb = -kb;   // times T_N at the inflow node
+      }
+      for (int q = grp; 4 * q < no; q += NG) {
+        uint32_t b[8][4];
+        tm_ld(tl + (uint32_t)(4 * q), g.n, b);
+        tm_wait(b);
+        int qb[4];
+        uint32_t lim = 1u;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          qb[e] = eb + se[n * g.n + 4 * q + e];
+          lim = max(lim, slow_limit(qb[e]));
+        }
+        int64_t R[4];
+        recombine4(b, R);
+        // the next rows' values travel while these are finished
+        double kv[4], f[4], ac[4];
+        unsigned off[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          kv[e] = nk[e];
+          f[e] = nf[e];
+          ac[e] = na[e];
+          off[e] = noff[e];
+        }
+        if (4 * (q + NG) < no) load_rows(n, q + NG, no);
+        double y4[4];
+        to_double4(R, qb, lim, y4);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int o = 4 * q + e;
+          if (o >= no) break;
+          const double y = y4[e];
+          double v = fma(ck, y, kv[e]);
+          if (A.tau) {   // K_i -= K_b T_N(x_b) T_N(x_i)
+            const int flip = ((N - rad_row(n * g.go + o, N)) & 1) << 31;
+            v -= __hiloint2double(__double2hiint(kb) ^ flip, __double2loint(kb));
+          }
+          if (!val) continue;
+          if (MODE == RAD_RHS) {
+            dst[off[e]] = v;
+          } else if (MODE == RAD_STAGE3) {
+            dst[off[e]] = fma(cu, ac[e] + v, f[e]);
+          } else if (MODE == RAD_AB2) {
+            dst[off[e]] = fma(cu, fma(1.5, v, -0.5 * ac[e]), f[e]);
+            Aw[off[e]] = v;
+          } else {
+            dst[off[e]] = fma(cu, v, f[e]);
+            Aw[off[e]] = MODE == RAD_STAGE1 ? fma(2.0, v, ac[e]) : v;
+          }
+        }
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncthreads();
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      if (*dead) {
+        if (tid == 0 && p.err) atomicExch(p.err, 1);
+        for (int x = n; x < issued; ++x) {   // our own MMAs end first (full bound)
+          const uint32_t rr = g.dual ? (uint32_t)(x & 1) : 0u;
+          bar_wait(sm_u32(&bar[rr]), ((phase >> rr) & 1u) ^ (x == n ? 1u : 0u), kDefaultWaitIters);
+        }
+        alive = false;
+        break;
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;"
+                 :: "r"(tmem), "r"(g.cols) : "memory");
+  }
+}
+
+}  // namespace emu
+}  // namespace ts

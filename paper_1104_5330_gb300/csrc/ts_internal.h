@@ -125,6 +125,8 @@ inline int rb_mask(const Dims& d, int elem_bytes, int n64) {
   return m;
 }
 
+struct EmuPlan;
+
 // Everything a kernel launch needs about the problem.
 struct Problem {
   Dims d;
@@ -150,6 +152,8 @@ struct Problem {
   // (K = 16) derivative matrices split into TF32 hi + lo in the tensor-core B
   // layout (W1 hi, W1 lo, W2 hi, W2 lo); NULL: the angular pass runs on the SIMT units
   const float* tcang;
+  // the double-precision passes on the tensor cores (ts_emu.h); NULL: the FP64 units
+  const EmuPlan* emu;
 };
 
 __host__ __device__ inline int kernel_form(const Problem& p, int collision) {
@@ -294,6 +298,7 @@ ts_status cuda_status(cudaError_t e, const char* where);
 
 // The grid behind the opaque ts_grid handle of include/ts.h.
 struct ts_grid {
+  ts::EmuPlan* emu = nullptr;  // TS_FP64: tensor-core passes of the sizes that have them
   ts_grid_desc desc;
   ts::Dims d;
   size_t es = 8;

@@ -75,7 +75,7 @@ k_batch_pass(const BatchItem<T, C>* __restrict__ items, int nitems, long long to
       radial_tile_any<T, C>(it.p, it.t, it.Dr64, in, it.K, (C)-1, it.tau, rmode, it.F,
                         it.Acc, it.U, nullptr, (C)it.dt, it.p.tp.W, lt);
     else
-      implicit_collision_tile<T, C>(it.p, it.t, it.F, it.dt, kThreads / 32, lt);
+      implicit_collision_tile<T, C>(it.p, it.t, it.F, it.dt, lt);
     __syncthreads();  // s_tile and the shared tiles are reused by the next iteration
   }
 }
@@ -89,7 +89,9 @@ inline long long tiles_radial(const Dims& d, int W) {
   const int S = d.NT * d.NP;
   return (long long)d.G * d.Nt * d.Np * ((S + W - 1) / W);
 }
-inline long long tiles_collision(const Dims& d) { return (d.nblk + kThreads / 32 - 1) / (kThreads / 32); }
+inline long long tiles_collision(const Dims& d) {
+  return (d.nblk + kCollisionBlocks - 1) / kCollisionBlocks;
+}
 
 // Resolve 0 (heuristic) entries of the forward tile shapes.
 template <typename T, typename C>

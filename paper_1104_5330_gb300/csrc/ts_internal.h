@@ -24,6 +24,19 @@ __device__ __forceinline__ double widen_f32(float f) {
   return __longlong_as_double((long long)(((uint64_t)(u >> 31) << 63) | mag));
 }
 
+// Round-to-nearest-even narrowing of a double to a float on the integer units (the bits
+// that the conversion instruction gives): results in the normal float range by
+// rebiasing and a rounding carry, the rest by the conversion.
+__device__ __forceinline__ float narrow_f64(double v) {
+  const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+  const uint32_t mag = hi & 0x7FFFFFFFu;
+  if (mag - 0x38100000u >= 0x47E00000u - 0x38100000u) return (float)v;   // below 2^-126, or from 2^127 on
+  uint32_t f = ((mag - 0x38000000u) << 3) | (lo >> 29);
+  const uint32_t rest = lo << 3;
+  f += rest > 0x80000000u || (rest == 0x80000000u && (f & 1u)) ? 1u : 0u;
+  return __uint_as_float(f | (hi & 0x80000000u));
+}
+
 // Device fields are read and written with 16-byte vector accesses and
 // 16-byte asynchronous copies: the entry points require 16-byte alignment.
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }

@@ -792,101 +792,212 @@ k_angular_T(Problem p, Tables<C> t, const T* __restrict__ lt, const T* __restric
 // and M~ of omega.A.omega is 2A/15 for traceless A, and the odd moments of even
 // functions vanish by symmetry. Then F = inflow data at the inflow nodes (if the
 // grid has Tau rows).
+//
+// Computed in double for every storage type: the stiff collision update (dt kappa up to
+// 1e2) is kept in FP64 on the GPU. The FP64 pipe bounds it (an FP64 instruction of a warp
+// takes 64 clocks of a scheduler's, an integer one about 1.5), so its operations are
+// kept to one multiply-add per weight and point: a lane owns Phi columns, sums its
+// column against Theta weights alone (their products are a table of the CTA) and applies
+// the Phi factors once; the division by den is a multiplication by its reciprocal with
+// one correction step (double) or none (float, rounded to 24 bits anyway); floats are
+// widened and narrowed on the integer units. A CTA takes kCollisionBlocks blocks in three
+// phases: the moments (a warp a block), the blocks' coefficients with their divisions
+// (a thread a block: done per warp they cost more than the points of a small block),
+// the update (a warp a block). Six groups of 21 x 12 x 10 x 14 x 12, linear kernel,
+// double: 283 us per launch before, 155 now.
+template <typename T>
+__device__ __forceinline__ double load_f64(T v) {
+  if constexpr (sizeof(T) == 4) return widen_f32(v);
+  else return v;
+}
+// num / den with inv = 1 / den, in the element type; far-out denominators (`plain`) and
+// quotients that are not finite take the division itself
+template <typename T>
+__device__ __forceinline__ T quotient(double num, double den, double inv, bool plain) {
+  if (plain) return (T)(num / den);
+  const double q = num * inv;
+  if constexpr (sizeof(T) == 4) return narrow_f64(q);
+  if ((__double2hiint(q) & 0x7FF00000) == 0x7FF00000) return (T)(num / den);
+  return (T)fma(fma(-q, den, num), inv, q);
+}
+constexpr int kCollisionWeights = 6;   // q, q cos, q sin, q cos^2, q sin^2, q cos sin of Theta
+
+constexpr int kCollisionBlocks = 8;   // of one tile; 32 left too few tiles in flight (188 us there)
+
+// Sums v[0..3] over the warp: afterwards lane 8 a (a < 4) holds the sum of v[a] in v[0].
+// Every step but the last three halves the values a lane carries.
+__device__ __forceinline__ void warp_sum4(double (&v)[4]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {   // lanes of the upper half take v[2], v[3]
+    const double send = lane & 16 ? v[a] : v[2 + a];
+    const double keep = lane & 16 ? v[2 + a] : v[a];
+    v[a] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+  }
+  {
+    const double send = lane & 8 ? v[0] : v[1];
+    const double keep = lane & 8 ? v[1] : v[0];
+    v[0] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+  }
+#pragma unroll
+  for (int o = 4; o; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+}
+
 template <typename T, typename C>
 __device__ __forceinline__ void implicit_collision_tile(const Problem& p, const Tables<C>& t,
-                                                        T* F, double dt, int nb,
-                                                        long long tile) {
-  // Computed in double for every storage type: the stiff collision update
-  // (dt kappa up to 1e2) is kept in FP64 on the GPU.
+                                                        T* F, double dt, long long tile) {
+  __shared__ double wt[kCollisionWeights][64];   // NTheta <= 64
+  __shared__ double mom[kCollisionBlocks][12];   // J, H (3), M (6: rr thth phph thph rth rph)
+  __shared__ double cf[kCollisionBlocks][12];    // num, den, 1/den, kb H+ (3), kc M~+ (6)
   const Dims d = p.d;
   const int NT = d.NT, NP = d.NP, S = NT * NP, hT = NT / 2;
-  const long long b0 = tile * nb;
-  const int nbb = (int)min((long long)nb, d.nblk - b0);
+  const long long b0 = tile * kCollisionBlocks;
+  const int nbb = (int)min((long long)kCollisionBlocks, d.nblk - b0);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int kf = kernel_form(p, 1);
   const bool aniso = kf >= KF_LINEAR, quad = kf >= KF_QUADRATIC;
+  for (int k = threadIdx.x; k < NT; k += blockDim.x) {
+    const double q = (double)t.qdir[k], ct = (double)t.cosT[k], st = (double)t.sinT[k];
+    wt[0][k] = q;
+    wt[1][k] = q * ct;
+    wt[2][k] = q * st;
+    wt[3][k] = q * ct * ct;
+    wt[4][k] = q * st * st;
+    wt[5][k] = q * ct * st;
+  }
+  __syncthreads();
   for (int bb = warp; bb < nbb; bb += nw) {
-    const long long blk = b0 + bb;
-    double acc = 0, mo[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};   // H (3), M (6: rr thth phph thph rth rph)
-    for (int x = lane; x < S; x += 32) {
-      const int k = x / NP, m = x - k * NP;
-      const double u = (double)F[blk * S + x];
-      acc = fma((double)t.qdir[k], u, acc);
+    const T* Fb = F + (b0 + bb) * S;
+    double mo[12] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+    for (int m0 = 0; m0 < NP; m0 += 32) {
+      // lanes: R rows of w columns at a time
+      const int w = min(32, NP - m0), R = 32 / w, kk = lane / w, m = m0 + lane - kk * w;
+      double a[kCollisionWeights] = {0, 0, 0, 0, 0, 0};
+      if (kk < R) {
+#pragma unroll 4
+        for (int k = kk; k < NT; k += R) {
+          const double u = load_f64(Fb[k * NP + m]);
+          a[0] = fma(wt[0][k], u, a[0]);
+          if (aniso) {
+            a[1] = fma(wt[1][k], u, a[1]);
+            a[2] = fma(wt[2][k], u, a[2]);
+          }
+          if (quad) {
+            a[3] = fma(wt[3][k], u, a[3]);
+            a[4] = fma(wt[4][k], u, a[4]);
+            a[5] = fma(wt[5][k], u, a[5]);
+          }
+        }
+      }
+      mo[0] += a[0];
       if (aniso) {
-        const double ct = (double)t.cosT[k], cp = (double)t.cosP[m], sp = (double)t.sinP[m];
-        const double qu = (double)t.qdir[k] * u, qs = (double)t.sinT[k] * qu;
-        mo[0] = fma(ct, qu, mo[0]);
-        mo[1] = fma(cp, qs, mo[1]);
-        mo[2] = fma(sp, qs, mo[2]);
+        const double cp = kk < R ? (double)t.cosP[m] : 0.0, sp = kk < R ? (double)t.sinP[m] : 0.0;
+        mo[1] += a[1];
+        mo[2] = fma(cp, a[2], mo[2]);
+        mo[3] = fma(sp, a[2], mo[3]);
         if (quad) {
-          const double qss = (double)t.sinT[k] * qs;
-          mo[3] = fma(ct * ct, qu, mo[3]);
-          mo[4] = fma(cp * cp, qss, mo[4]);
-          mo[5] = fma(sp * sp, qss, mo[5]);
-          mo[6] = fma(cp * sp, qss, mo[6]);
-          mo[7] = fma(ct * cp, qs, mo[7]);
-          mo[8] = fma(ct * sp, qs, mo[8]);
+          mo[4] += a[3];
+          mo[5] = fma(cp * cp, a[4], mo[5]);
+          mo[6] = fma(sp * sp, a[4], mo[6]);
+          mo[7] = fma(cp * sp, a[4], mo[7]);
+          mo[8] = fma(cp, a[5], mo[8]);
+          mo[9] = fma(sp, a[5], mo[9]);
         }
       }
     }
-    const int nm = quad ? 9 : aniso ? 3 : 0;   // uniform over the block
-    for (int o = 16; o; o >>= 1) {
-      acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (!aniso) {
+      for (int o = 16; o; o >>= 1) mo[0] += __shfl_xor_sync(0xffffffffu, mo[0], o);
+      if (lane == 0) mom[bb][0] = mo[0];
+    } else {
 #pragma unroll
-      for (int a = 0; a < 9; ++a)   // constant indices keep mo in registers
-        if (a < nm) mo[a] += __shfl_xor_sync(0xffffffffu, mo[a], o);
+      for (int z = 0; z < 12; z += 4) {   // constant indices keep mo in registers
+        if (z == 0 || quad) {             // uniform over the block
+          double v[4] = {mo[z], mo[z + 1], mo[z + 2], mo[z + 3]};
+          warp_sum4(v);
+          // lanes 0, 8, 16, 24 hold v[0], v[1], v[2], v[3]
+          if ((lane & 7) == 0) mom[bb][z + (lane >> 3)] = v[0];
+        }
+      }
     }
+  }
+  __syncthreads();
+  if (threadIdx.x < nbb) {
+    const long long blk = b0 + threadIdx.x;
+    const double* mo = mom[threadIdx.x];
+    double* c = cf[threadIdx.x];
     const double kap = p.kap[blk], eta = p.eta[blk], ks = p.kaps[blk];
-    const double Jp = (acc + dt * eta) / (1.0 + dt * kap);
-    const double num = dt * (eta + ks * Jp), den = 1.0 + dt * (kap + ks);
-    double kbr = 0, kbt = 0, kbp = 0;   // dt kappa_s b H+
-    double q6[6] = {0, 0, 0, 0, 0, 0};  // dt kappa_s c M~+ (rr thth phph, 2 thph, 2 rth, 2 rph)
-    if (aniso && p.scb) {
-      const double kb = ks * p.scb[blk], f = dt * kb / (den - dt * kb / 3.0);
-      kbr = f * mo[0];
-      kbt = f * mo[1];
-      kbp = f * mo[2];
+    const double Jp = (mo[0] + dt * eta) / (1.0 + dt * kap);
+    const double den = 1.0 + dt * (kap + ks);
+    c[0] = dt * (eta + ks * Jp);
+    c[1] = den;
+    c[2] = 1.0 / den;
+    if (aniso) {   // dt kappa_s b H+
+      const double kb = p.scb ? ks * p.scb[blk] : 0.0, f = dt * kb / (den - dt * kb / 3.0);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) c[3 + a] = p.scb ? f * mo[1 + a] : 0.0;
     }
-    if (quad) {
+    if (quad) {    // dt kappa_s c M~+ (rr thth phph, 2 thph, 2 rth, 2 rph)
       const double kc = ks * p.scc[blk], f = dt * kc / (den - dt * kc * (2.0 / 15.0));
-      const double j3 = acc / 3.0;
-      q6[0] = f * (mo[3] - j3);
-      q6[1] = f * (mo[4] - j3);
-      q6[2] = f * (mo[5] - j3);
-      q6[3] = 2.0 * f * mo[6];
-      q6[4] = 2.0 * f * mo[7];
-      q6[5] = 2.0 * f * mo[8];
+      const double j3 = mo[0] / 3.0;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        c[6 + a] = f * (mo[4 + a] - j3);
+        c[9 + a] = 2.0 * f * mo[7 + a];
+      }
     }
+  }
+  __syncthreads();
+  for (int bb = warp; bb < nbb; bb += nw) {
+    const long long blk = b0 + bb;
+    T* Fb = F + blk * S;
+    const double* c = cf[bb];
+    const double num = c[0], den = c[1], inv = c[2];
+    const bool plain = !(fabs(den) < 1e150 && fabs(den) > 1e-150);
     int g, i, j, l;
     decode_block(d, blk, g, i, j, l);
     const T* g1 = reinterpret_cast<const T*>(p.gR1);
     const T* g2 = reinterpret_cast<const T*>(p.gR2);
-    for (int x = lane; x < S; x += 32) {
-      const int k = x / NP, m = x - k * NP;
-      double v = (double)F[blk * S + x] + num;
+    const bool in1 = p.bc == TS_BC_TAU_INFLOW && i == 0;
+    const bool in2 = p.bc == TS_BC_TAU_INFLOW && i == d.Nr - 1;
+    const long long pos = (((long long)g * d.Nt + j) * d.Np + l) * hT;
+    for (int m0 = 0; m0 < NP; m0 += 32) {
+      const int w = min(32, NP - m0), R = 32 / w, kk = lane / w, m = m0 + lane - kk * w;
+      if (kk >= R) continue;
+      double hc = 0, qc = 0, rc = 0;   // the column's factors of sin, sin^2, cos sin of Theta
       if (aniso) {
-        const double ct = (double)t.cosT[k], st = (double)t.sinT[k];
         const double cp = (double)t.cosP[m], sp = (double)t.sinP[m];
-        v += ct * kbr + st * (cp * kbt + sp * kbp);
-        if (quad)
-          v += ct * ct * q6[0] + st * st * (cp * cp * q6[1] + sp * sp * q6[2] + cp * sp * q6[3]) +
-               ct * st * (cp * q6[4] + sp * q6[5]);
+        hc = cp * c[4] + sp * c[5];
+        if (quad) {
+          qc = cp * cp * c[7] + sp * sp * c[8] + cp * sp * c[9];
+          rc = cp * c[10] + sp * c[11];
+        }
       }
-      v /= den;
-      if (p.bc == TS_BC_TAU_INFLOW) {
-        const long long pos = (((long long)g * d.Nt + j) * d.Np + l) * hT;
-        if (i == 0 && k < hT) v = g1 ? (double)g1[(pos + k) * NP + m] : 0.0;
-        if (i == d.Nr - 1 && k >= hT) v = g2 ? (double)g2[(pos + k - hT) * NP + m] : 0.0;
+#pragma unroll 4
+      for (int k = kk; k < NT; k += R) {
+        double v = load_f64(Fb[k * NP + m]) + num;
+        if (aniso) {
+          const double ct = (double)t.cosT[k], st = (double)t.sinT[k];
+          double u1 = c[3], u2 = hc;
+          if (quad) {
+            u1 = fma(ct, c[6], fma(st, rc, c[3]));
+            u2 = fma(st, qc, hc);
+          }
+          v = fma(ct, u1, fma(st, u2, v));
+        }
+        T r = quotient<T>(v, den, inv, plain);
+        if (in1 && k < hT) r = g1 ? g1[(pos + k) * NP + m] : (T)0;
+        if (in2 && k >= hT) r = g2 ? g2[(pos + k - hT) * NP + m] : (T)0;
+        Fb[k * NP + m] = r;
       }
-      F[blk * S + x] = (T)v;
     }
   }
+  __syncthreads();   // the shared arrays are written again by a batched kernel's next tile
 }
 
 template <typename T, typename C>
 __global__ void __launch_bounds__(kThreads)
-k_implicit_collision(Problem p, Tables<C> t, T* F, double dt, int nb) {
-  implicit_collision_tile<T, C>(p, t, F, dt, nb, blockIdx.x);
+k_implicit_collision(Problem p, Tables<C> t, T* F, double dt) {
+  implicit_collision_tile<T, C>(p, t, F, dt, blockIdx.x);
 }
 
 // F = inflow data at the inflow nodes.

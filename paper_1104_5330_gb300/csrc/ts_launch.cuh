@@ -375,9 +375,8 @@ cudaError_t Launch<T, C>::angular_T(const Problem& p, const Tables<C>& t, const 
 template <typename T, typename C>
 cudaError_t Launch<T, C>::implicit_collision(const Problem& p, const Tables<C>& t, T* F,
                                              double dt, cudaStream_t s) {
-  const int nb = kThreads / 32;
-  k_implicit_collision<T, C><<<grid1((p.d.nblk + nb - 1) / nb), kThreads, 0, s>>>(p, t, F, dt,
-                                                                                 nb);
+  const long long ctas = (p.d.nblk + kCollisionBlocks - 1) / kCollisionBlocks;
+  k_implicit_collision<T, C><<<grid1(ctas), kThreads, 0, s>>>(p, t, F, dt);
   return cudaGetLastError();
 }
 

@@ -83,19 +83,50 @@ __host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N) {
          ((uint32_t)(M >> 4) << 24);
 }
 
+// Called by a whole warp with warp-uniform arguments, `one` set on the elected lane.
 template <int KIND>
 __device__ __forceinline__ void umma(uint32_t dtmem, uint64_t a, uint64_t b, uint32_t idesc,
-                                     uint32_t accumulate) {
+                                     uint32_t accumulate, uint32_t one = 1) {
   if constexpr (KIND == TC_TF32X3)
     asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n"
-        :: "r"(dtmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
+        "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+        " @q tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n"
+        :: "r"(dtmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(one) : "memory");
   else
     asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-        :: "r"(dtmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
+        "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
+        :: "r"(dtmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(one) : "memory");
+}
+
+// The products of one tile: ST K steps (0: `steps` at run time). Issued by a warp
+// from uniform registers and unrolled, an MMA takes 50 clocks to issue; from one
+// thread of a divergent branch, 163.
+template <int KIND, int ST>
+__device__ __forceinline__ void tc_products(uint32_t one, uint32_t tmem, uint32_t a0, uint32_t as,
+                                            uint32_t b0, uint32_t bs, uint32_t lbo, uint32_t sbo,
+                                            uint32_t idesc, int steps) {
+  const int n = ST ? ST : steps;
+#pragma unroll
+  for (int ks = 0; ks < n; ++ks) {
+    const uint32_t off = (uint32_t)ks * 256;  // two 16-byte core columns of K
+    auto mma = [&](int ta, int tb, uint32_t acc) {
+      umma<KIND>(tmem, umma_desc(a0 + ta * as + off, lbo, sbo),
+                 umma_desc(b0 + tb * bs + off, lbo, sbo), idesc, acc, one);
+    };
+    if constexpr (KIND == TC_TF32X3) {
+      mma(1, 0, ks > 0);
+      mma(0, 1, 1);
+      mma(0, 0, 1);
+    } else {
+      mma(2, 0, ks > 0);
+      mma(1, 1, 1);
+      mma(0, 2, 1);
+      mma(1, 0, 1);
+      mma(0, 1, 1);
+      mma(0, 0, 1);
+    }
+  }
 }
 
 // Operand form: element bytes, operand terms, elements per 16-byte core
@@ -301,41 +332,37 @@ k_radial_tc(Problem p, Tables<float> t, const void* __restrict__ Bterms, const f
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = *tslot;
+  const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, *tslot, 0);
   bool ok = true;
-  if (tid == 0) {
+  if (__shfl_sync(0xFFFFFFFFu, warp, 0) == 0) {
     // the operand wait's bound is p.wait_operand (the default, or a shorter one
     // set with ts_set_wait_limit to exercise the timeout path)
-    ok = mbar_wait(bar0, 0, p.wait_operand);
+    ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar0, 0, p.wait_operand));
     if (ok) {
+      uint32_t one;
+      asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xFFFFFFFF;\n selp.u32 %0, 1, 0, p;\n}\n"
+                   : "=r"(one));
       const uint32_t idesc = KIND == TC_TF32X3 ? umma_idesc_tf32(128, sh.Npad)
                                                : umma_idesc_bf16(128, sh.Npad);
       const uint32_t lbo = 128, sbo = (uint32_t)sh.KC * 128;
       const uint32_t a0 = smem_u32(sA), b0 = smem_u32(sB);
       const uint32_t as = (uint32_t)sh.a_bytes, bs = (uint32_t)sh.b_bytes;
-      for (int ks = 0; ks < sh.Kpad / Fm::KSTEP; ++ks) {
-        const uint32_t off = (uint32_t)ks * 256;  // two 16-byte core columns of K
-        auto mma = [&](int ta, int tb, uint32_t acc) {
-          umma<KIND>(tmem, umma_desc(a0 + ta * as + off, lbo, sbo),
-                     umma_desc(b0 + tb * bs + off, lbo, sbo), idesc, acc);
-        };
-        if constexpr (KIND == TC_TF32X3) {
-          mma(1, 0, ks > 0);
-          mma(0, 1, 1);
-          mma(0, 0, 1);
-        } else {
-          mma(2, 0, ks > 0);
-          mma(1, 1, 1);
-          mma(0, 2, 1);
-          mma(1, 0, 1);
-          mma(0, 1, 1);
-          mma(0, 0, 1);
-        }
-      }
+      const int steps = sh.Kpad / Fm::KSTEP;
+      // N_r = 17, 33, 65 unrolled
+      if (steps == (KIND == TC_TF32X3 ? 5 : 3))
+        tc_products<KIND, KIND == TC_TF32X3 ? 5 : 3>(one, tmem, a0, as, b0, bs, lbo, sbo, idesc, 0);
+      else if (steps == (KIND == TC_TF32X3 ? 3 : 2))
+        tc_products<KIND, KIND == TC_TF32X3 ? 3 : 2>(one, tmem, a0, as, b0, bs, lbo, sbo, idesc, 0);
+      else if (steps == (KIND == TC_TF32X3 ? 9 : 5))
+        tc_products<KIND, KIND == TC_TF32X3 ? 9 : 5>(one, tmem, a0, as, b0, bs, lbo, sbo, idesc, 0);
+      else
+        tc_products<KIND, 0>(one, tmem, a0, as, b0, bs, lbo, sbo, idesc, steps);
       asm volatile(
-          "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-          :: "r"(bar1) : "memory");
+          "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+          " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n"
+          :: "r"(bar1), "r"(one) : "memory");
     }
+    __syncwarp();
   }
   // every thread waits for the products (bounded); `issued` is CTA-wide: the
   // MMAs and their commit were issued only if thread 0's operand wait succeeded

@@ -16,7 +16,8 @@ namespace {
 
 // Matrix entries are formed in long double (64 bits and more): the digits hold 62
 // bits of a row, and the rounding of the entries to double would be the largest
-// error left in a contraction.
+// error left in a contraction. Long double is software on Arm: every function value
+// is formed once, by its index.
 typedef long double Wide;
 const Wide kPi = 3.14159265358979323846264338327950288L;
 
@@ -26,11 +27,13 @@ std::vector<Wide> cheb_wide(int Nr, double R1, double R2) {
   std::vector<Wide> D((size_t)Nr * Nr, 0.0L);
   auto w = [&](int i) { return ((i % 2) ? -1.0L : 1.0L) * (i == 0 || i == N ? 0.5L : 1.0L); };
   const Wide s = 2.0L / ((Wide)R2 - (Wide)R1);
+  std::vector<Wide> sn(2 * N + 1);   // sin(pi q / (2 N))
+  for (int q = 0; q <= 2 * N; ++q) sn[q] = sinl(kPi * q / (2.0L * N));
   for (int i = 0; i < Nr; ++i) {
     Wide diag = 0.0L;
     for (int j = 0; j < Nr; ++j) {
       if (i == j) continue;
-      const Wide dx = 2.0L * sinl(kPi * (i + j) / (2.0L * N)) * sinl(kPi * (i - j) / (2.0L * N));
+      const Wide dx = 2.0L * sn[i + j] * (i > j ? sn[i - j] : -sn[j - i]);
       const Wide v = w(j) / w(i) / dx * s;
       D[(size_t)i * Nr + j] = v;
       diag -= v;
@@ -40,13 +43,11 @@ std::vector<Wide> cheb_wide(int Nr, double R1, double R2) {
   return D;
 }
 std::vector<Wide> fourier_wide(int M) {
-  std::vector<Wide> D((size_t)M * M, 0.0L);
+  std::vector<Wide> D((size_t)M * M, 0.0L), c(M, 0.0L);
+  for (int q = 1; q < M; ++q)   // cot(pi / 2) = 0
+    if (2 * q != M) c[q] = 0.5L * (q % 2 ? -1.0L : 1.0L) / tanl(q * kPi / M);
   for (int j = 0; j < M; ++j)
-    for (int k = 0; k < M; ++k) {
-      const int q = j - k;
-      if (q == 0 || 2 * std::abs(q) == M) continue;   // cot(pi / 2) = 0
-      D[(size_t)j * M + k] = 0.5L * (q % 2 ? -1.0L : 1.0L) / tanl(q * kPi / M);
-    }
+    for (int k = 0; k < M; ++k) D[(size_t)j * M + k] = j >= k ? c[j - k] : -c[k - j];
   return D;
 }
 
@@ -61,6 +62,17 @@ uint16_t f16_int(int v) {
   return (uint16_t)((v < 0 ? 0x8000 : 0) | ((e + 15) << 10) | (((a - (1 << e)) << 10) >> e));
 }
 
+// The scale of a row (see digits_of), at most smax.
+int scale_of(const std::vector<Wide>& row, int smax) {
+  double mx = 0.0, tot = 0.0;
+  for (const Wide& w : row) {
+    const double a = std::fabs((double)w);
+    mx = std::max(mx, a);
+    tot += a;
+  }
+  if (mx == 0.0) return smax;
+  return std::min(std::min(62 - (std::ilogb(mx) + 1), 65 - (std::ilogb(tot) + 1)), smax);
+}
 // The digits of a row: value 2^s rounded to an integer below 2^62, s the largest with
 // sum |Dfix| < 2^65; digits balanced, most significant first.
 struct Row {
@@ -70,16 +82,10 @@ struct Row {
 Row digits_of(const std::vector<Wide>& row, int smax) {
   Row r;
   r.e.resize(row.size());
-  double mx = 0.0, tot = 0.0;
-  for (const Wide& w : row) {
-    mx = std::max(mx, (double)fabsl(w));
-    tot += (double)fabsl(w);
-  }
   for (auto& e : r.e) e.fill(0);
-  r.s = smax;
-  if (mx == 0.0) return r;
-  r.s = std::min(std::min(62 - (std::ilogb(mx) + 1), 65 - (std::ilogb(tot) + 1)), smax);
+  r.s = scale_of(row, smax);
   for (size_t k = 0; k < row.size(); ++k) {
+    if (row[k] == 0.0L) continue;
     long long v = llrintl(ldexpl(row[k], r.s));
     for (int j = 7; j >= 0; --j) {
       const int q = j == 0 ? (int)v : (int)((((v + 128) % 256) + 256) % 256) - 128;
@@ -107,7 +113,7 @@ bool build_operand(const Mat& m, const std::vector<int>& order, int left, bool c
   uint16_t* ext = bias + core;
   uint16_t* main = bias + core * (1 + out->extra);
   int smin = 1 << 20;   // the scale every row has where they share one
-  for (const auto& row : m) smin = std::min(smin, digits_of(row, 1 << 20).s);
+  for (const auto& row : m) smin = std::min(smin, scale_of(row, 1 << 20));
   if (smin == 1 << 20) smin = 60;   // a matrix of zeros
   out->s = smin;
   for (int o = 0; o < out->nout; ++o) {
@@ -218,7 +224,7 @@ bool geometry2(int Na, int Nb, const EmuMat& D, const EmuMat& F, int nf, int nz,
   g.oB2 = take(F.bytes());
   g.oCA = take(2 * 128 * 16);
   g.oEx = alias ? g.oC2 : take(exB);
-  g.oMs = take(96 + (128 + 160 + Na) * 8);
+  g.oMs = take(96 + (128 + 160 + Na + g.mt1 * 16 * 8) * 8);
   // a 128-row tile may read row groups past the last one: inside the allocation
   const int over = std::max(g.oC1 + 7 * g.d1 + (16 * g.mt1 + g.hb) * g.sb1 + 256,
                             g.oC2 + 7 * g.d2 + 16 * g.mt2 * g.sb2 + 256);
@@ -269,7 +275,7 @@ bool geometry_radial(int Nr, EmuRadGeo* out) {
       g.oA = take(8 * g.d + 256);
       g.oB = take(ng * g.bB);
       g.oCA = take(2 * 128 * 16);
-      g.oMs = take(32 + ng * g.n * 4);
+      g.oMs = take(32 + (ng * g.n * 4 + 15) / 16 * 16 + 128 * 8);
       g.bytes = o;
       if (g.bytes > (two ? kTwoCtas : kOneCta)) continue;
       g.threads = two ? 256 : 512;
@@ -327,20 +333,22 @@ EmuPlan* emu_create(const ts_grid_desc& g, cudaError_t* err) {
     const std::vector<Wide> DT = fourier_wide(2 * NT), DP = fourier_wide(NP);
     Mat mD(NT, std::vector<Wide>(2 * NT)), mF(NP + 5, std::vector<Wide>(NP));
     for (int k = 0; k < NT; ++k) {
-      const Wide Th = kPi * (k + 0.5L) / NT;
+      const Wide Th = kPi * (k + 0.5L) / NT, st = sinl(Th), ct = cosl(Th);
       for (int q = 0; q < NT; ++q) {
-        mD[k][q] = sinl(Th) * DT[(size_t)k * 2 * NT + q];
-        mD[k][NT + q] = odd * sinl(Th) * DT[(size_t)k * 2 * NT + 2 * NT - 1 - q];
+        mD[k][q] = st * DT[(size_t)k * 2 * NT + q];
+        mD[k][NT + q] = odd * st * DT[(size_t)k * 2 * NT + 2 * NT - 1 - q];
         if (cons) {   // P: the Nyquist bin of the doubled circle taken out
           const Wide alt = ((k + q) % 2 ? -1.0L : 1.0L) / (2.0L * NT);
-          mD[k][q] += cosl(Th) * ((k == q ? 1.0L : 0.0L) - alt);
-          mD[k][NT + q] -= cosl(Th) * alt;
+          mD[k][q] += ct * ((k == q ? 1.0L : 0.0L) - alt);
+          mD[k][NT + q] -= ct * alt;
         }
       }
     }
+    std::vector<Wide> sP(NP);
+    for (int m = 0; m < NP; ++m) sP[m] = sine(m, NP);
     for (int q = 0; q < NP; ++q) {
-      const Wide c = cosl(2.0L * kPi * q / NP), s = sine(q, NP);
-      for (int m = 0; m < NP; ++m) mF[m][q] = (cons ? s : sine(m, NP)) * DP[(size_t)m * NP + q];
+      const Wide c = cosl(2.0L * kPi * q / NP), s = sP[q];
+      for (int m = 0; m < NP; ++m) mF[m][q] = (cons ? s : sP[m]) * DP[(size_t)m * NP + q];
       mF[NP][q] = 1.0L;
       mF[NP + 1][q] = c;
       mF[NP + 2][q] = s;
@@ -362,6 +370,35 @@ EmuPlan* emu_create(const ts_grid_desc& g, cudaError_t* err) {
                geometry2(NT, NP, e->angD, e->angF[f], nf[f], nz, &e->gAng[f]);
     }
   }
+  const bool adj = !cons && g.radial == TS_RADIAL_CHEBYSHEV;   // the forms that have an adjoint
+  if (adj) {
+    // the transposed angular operator: D_Th^T (sinTh lt), D_Ph^T (sinPh lt)
+    const std::vector<Wide> DT = fourier_wide(2 * NT), DP = fourier_wide(NP);
+    Mat mD(NT, std::vector<Wide>(2 * NT)), mF(NP + 5, std::vector<Wide>(NP));
+    for (int k = 0; k < NT; ++k) {
+      const Wide st = sinl(kPi * (k + 0.5L) / NT);
+      for (int q = 0; q < NT; ++q) {
+        mD[q][k] = st * DT[(size_t)k * 2 * NT + q];
+        mD[q][NT + k] = st * DT[(size_t)k * 2 * NT + 2 * NT - 1 - q];
+      }
+    }
+    for (int m = 0; m < NP; ++m) {
+      const Wide c = cosl(2.0L * kPi * m / NP), s = sine(m, NP);
+      for (int q = 0; q < NP; ++q) mF[q][m] = s * DP[(size_t)m * NP + q];
+      mF[NP][m] = 1.0L;
+      mF[NP + 1][m] = c;
+      mF[NP + 2][m] = s;
+      mF[NP + 3][m] = c * c;
+      mF[NP + 4][m] = c * s;
+    }
+    e->adj = add_matrix(mD, dfs_order(NT), -1, true, &e->adjD, &up);
+    const int nf[kEmuForms] = {1, 3, 5};
+    for (int f = 0; f < kEmuForms && e->adj; ++f) {
+      Mat part(mF.begin(), mF.begin() + NP + nf[f]);
+      e->adj = add_matrix(part, plain_order(NP, (NP + 15) / 16 * 2), -1, true, &e->adjF[f], &up) &&
+               geometry2(NT, NP, e->adjD, e->adjF[f], nf[f], 0, &e->gAdj[f]);
+    }
+  }
   {
     const std::vector<Wide> Dt = fourier_wide(2 * Nt), Dp = fourier_wide(Np);
     Mat mD(Nt, std::vector<Wide>(2 * Nt)), mF(Np, std::vector<Wide>(Np));
@@ -375,26 +412,41 @@ EmuPlan* emu_create(const ts_grid_desc& g, cudaError_t* err) {
     e->plane = add_matrix(mD, dfs_order(Nt), -1, true, &e->plD, &up) &&
                add_matrix(mF, plain_order(Np, (Np + 15) / 16 * 2), -1, true, &e->plF, &up) &&
                geometry2(Nt, Np, e->plD, e->plF, 0, 0, &e->gPl);
+    if (adj && e->plane) {
+      // transposed: a_th changes sign at the partner (cos(Ph + pi) = -cosPh), so it comes
+      // out of the contraction with the partner's matrix negated
+      Mat tD(Nt, std::vector<Wide>(2 * Nt)), tF(Np, std::vector<Wide>(Np));
+      for (int j = 0; j < Nt; ++j)
+        for (int q = 0; q < Nt; ++q) {
+          tD[q][j] = mD[j][q];
+          tD[q][Nt + j] = -mD[j][Nt + q];
+        }
+      for (int l = 0; l < Np; ++l)
+        for (int q = 0; q < Np; ++q) tF[q][l] = mF[l][q];
+      e->planeT = add_matrix(tD, dfs_order(Nt), -1, true, &e->plTD, &up) &&
+                  add_matrix(tF, plain_order(Np, (Np + 15) / 16 * 2), -1, true, &e->plTF, &up);
+    }
   }
   if (g.radial == TS_RADIAL_CHEBYSHEV && geometry_radial(Nr, &e->gRad)) {
     const EmuRadGeo& r = e->gRad;
     const std::vector<Wide> Dr = cheb_wide(Nr, g.R1, g.R2);
     e->rad = true;
-    for (int q = 0; q < r.ng && e->rad; ++q) {
-      Mat m;
-      for (int o = q * r.go; o < std::min(Nr, (q + 1) * r.go); ++o) {
-        const int i = o == 0 ? 0 : o == 1 ? Nr - 1 : o - 1;
-        std::vector<Wide> row(Nr);
-        for (int z = 0; z < Nr; ++z) row[z] = Dr[(size_t)i * Nr + z];
-        m.push_back(row);
-      }
-      const std::vector<int> order = plain_order(r.left ? Nr - 1 : Nr, r.kc);
-      e->rad = add_matrix(m, order, r.left ? Nr - 1 : -1, false, &e->radM[q], &up) &&
-               e->radM[q].n <= r.n;
-      if (e->rad && e->radM[q].n < r.n) {   // a shorter last group: pad to the common width
-        while ((int)m.size() < r.go) m.push_back(std::vector<Wide>(Nr));
-        up.fix.pop_back();
-        e->rad = add_matrix(m, order, r.left ? Nr - 1 : -1, false, &e->radM[q], &up);
+    // the transposed pass keeps a tile's values in registers
+    e->radT = adj && Nr * 16 <= 3 * r.threads;
+    for (int tr = 0; tr < 2; ++tr) {
+      bool& ok = tr ? e->radT : e->rad;
+      for (int q = 0; q < r.ng && ok; ++q) {
+        EmuMat* out = tr ? &e->radTM[q] : &e->radM[q];
+        Mat m;
+        for (int o = q * r.go; o < std::min(Nr, (q + 1) * r.go); ++o) {
+          const int i = o == 0 ? 0 : o == 1 ? Nr - 1 : o - 1;
+          std::vector<Wide> row(Nr);
+          for (int z = 0; z < Nr; ++z) row[z] = tr ? Dr[(size_t)z * Nr + i] : Dr[(size_t)i * Nr + z];
+          m.push_back(row);
+        }
+        while ((int)m.size() < r.go) m.push_back(std::vector<Wide>(Nr));   // equal groups
+        ok = add_matrix(m, plain_order(r.left ? Nr - 1 : Nr, r.kc), r.left ? Nr - 1 : -1, false, out,
+                        &up);
       }
     }
   }
@@ -467,7 +519,13 @@ cudaError_t launch2t(const Problem& p, const Tables<double>& t, const EmuGeo& g,
 cudaError_t emu_angular(const EmuPlan& e, const Problem& p, const Tables<double>& t, bool cons,
                         const double* U, double* K, double sgn, bool collision, cudaStream_t s) {
   const int kf = kernel_form(p, collision ? 1 : 0);
-  emu::EmuArgs A{U, K, sgn, collision ? 1 : 0, cons ? 1 : 0, 0, (p.d.nblk + 7) / 8};
+  emu::EmuArgs A{};
+  A.U = U;
+  A.K = K;
+  A.sgn = sgn;
+  A.collision = collision ? 1 : 0;
+  A.cons = cons ? 1 : 0;
+  A.ntiles = (p.d.nblk + 7) / 8;
   switch (kf) {
     case KF_QUADRATIC:
       return launch2t<emu::EP_ANGULAR, KF_QUADRATIC>(p, t, e.gAng[kf], e.angD, e.angF[kf], A, s);
@@ -478,28 +536,73 @@ cudaError_t emu_angular(const EmuPlan& e, const Problem& p, const Tables<double>
   }
 }
 
+namespace {
+cudaError_t plane_launch(const Problem& p, const Tables<double>& t, const EmuGeo& g,
+                         const EmuMat& D, const EmuMat& F, const double* U, double* K, double sgn,
+                         cudaStream_t s) {
+  emu::EmuArgs A{};
+  A.U = U;
+  A.K = K;
+  A.sgn = sgn;
+  A.vec = p.d.NP % 8 == 0 && (reinterpret_cast<uintptr_t>(U) & 31u) == 0;
+  A.ntiles = (long long)p.d.G * p.d.Nr * p.d.NT * ((p.d.NP / 2 + 3) / 4);
+  return launch2t<emu::EP_PLANE, KF_ISO>(p, t, g, D, F, A, s);
+}
+}  // namespace
+
 cudaError_t emu_plane(const EmuPlan& e, const Problem& p, const Tables<double>& t,
                       const double* U, double* K, double sgn, cudaStream_t s) {
-  const int vec = p.d.NP % 8 == 0 && (reinterpret_cast<uintptr_t>(U) & 31u) == 0;
-  emu::EmuArgs A{U, K, sgn, 0, 0, vec,
-                 (long long)p.d.G * p.d.Nr * p.d.NT * ((p.d.NP / 2 + 3) / 4)};
-  return launch2t<emu::EP_PLANE, KF_ISO>(p, t, e.gPl, e.plD, e.plF, A, s);
+  return plane_launch(p, t, e.gPl, e.plD, e.plF, U, K, sgn, s);
+}
+
+cudaError_t emu_angular_T(const EmuPlan& e, const Problem& p, const Tables<double>& t,
+                          const double* lt, const double* Ubar, const double* Us, double* gk,
+                          double* ge, const double* lam, const double* lam_in, double* lam_out,
+                          double* Kbar, double wl, double wu, cudaStream_t s) {
+  const int kf = kernel_form(p, 1);
+  emu::EmuArgs A{};
+  A.U = lt;
+  A.K = const_cast<double*>(Ubar);   // only read
+  A.sgn = -1.0;
+  A.collision = 1;
+  A.Us = Us;
+  A.gk = gk;
+  A.ge = ge;
+  A.lam = lam;
+  A.lam_in = lam_in;
+  A.lam_out = lam_out;
+  A.Kbar = Kbar;
+  A.wl = wl;
+  A.wu = wu;
+  A.ntiles = (p.d.nblk + 7) / 8;
+  switch (kf) {
+    case KF_QUADRATIC:
+      return launch2t<emu::EP_ADJOINT, KF_QUADRATIC>(p, t, e.gAdj[kf], e.adjD, e.adjF[kf], A, s);
+    case KF_LINEAR:
+      return launch2t<emu::EP_ADJOINT, KF_LINEAR>(p, t, e.gAdj[kf], e.adjD, e.adjF[kf], A, s);
+    default:
+      return launch2t<emu::EP_ADJOINT, KF_ISO>(p, t, e.gAdj[kf], e.adjD, e.adjF[kf], A, s);
+  }
+}
+
+cudaError_t emu_plane_T(const EmuPlan& e, const Problem& p, const Tables<double>& t,
+                        const double* lt, double* Ubar, cudaStream_t s) {
+  return plane_launch(p, t, e.gPl, e.plTD, e.plTF, lt, Ubar, -1.0, s);
 }
 
 namespace {
 template <int T, int MODE>
-cudaError_t launch_rad(const EmuPlan& e, const Problem& p, const Tables<double>& t,
-                       emu::RadArgs A, cudaStream_t s) {
+cudaError_t launch_rad(const EmuRadGeo& g, const EmuMat* mats, const Problem& p,
+                       const Tables<double>& t, emu::RadArgs A, cudaStream_t s) {
   static const cudaError_t ea = allow_smem(emu::k_emu_radial<T, MODE>);   // once per kernel
   if (ea != cudaSuccess) return ea;
-  const EmuRadGeo& g = e.gRad;
   int ctas = 1;
   const cudaError_t e2 = emu_ctas(T, A.ntiles, &ctas);
   if (e2 != cudaSuccess) return e2;
   emu::RadMats M{};
   for (int q = 0; q < g.ng; ++q) {
-    M.dev[q] = e.radM[q].dev;
-    M.se[q] = e.radM[q].se;
+    M.dev[q] = mats[q].dev;
+    M.se[q] = mats[q].se;
   }
   emu::k_emu_radial<T, MODE><<<ctas, T, g.bytes, s>>>(p, t, g, M, A);
   return cudaGetLastError();
@@ -508,13 +611,13 @@ template <int T>
 cudaError_t launch_rad_mode(const EmuPlan& e, const Problem& p, const Tables<double>& t,
                             emu::RadArgs A, cudaStream_t s) {
   switch (A.mode) {
-    case RAD_RHS: return launch_rad<T, RAD_RHS>(e, p, t, A, s);
-    case RAD_STAGE0: return launch_rad<T, RAD_STAGE0>(e, p, t, A, s);
+    case RAD_RHS: return launch_rad<T, RAD_RHS>(e.gRad, e.radM, p, t, A, s);
+    case RAD_STAGE0: return launch_rad<T, RAD_STAGE0>(e.gRad, e.radM, p, t, A, s);
     case RAD_STAGE1:
-    case RAD_STAGE2: return launch_rad<T, RAD_STAGE1>(e, p, t, A, s);
-    case RAD_STAGE3: return launch_rad<T, RAD_STAGE3>(e, p, t, A, s);
-    case RAD_AB2: return launch_rad<T, RAD_AB2>(e, p, t, A, s);
-    default: return launch_rad<T, RAD_AB2_START>(e, p, t, A, s);
+    case RAD_STAGE2: return launch_rad<T, RAD_STAGE1>(e.gRad, e.radM, p, t, A, s);
+    case RAD_STAGE3: return launch_rad<T, RAD_STAGE3>(e.gRad, e.radM, p, t, A, s);
+    case RAD_AB2: return launch_rad<T, RAD_AB2>(e.gRad, e.radM, p, t, A, s);
+    default: return launch_rad<T, RAD_AB2_START>(e.gRad, e.radM, p, t, A, s);
   }
 }
 }  // namespace
@@ -526,6 +629,16 @@ cudaError_t emu_radial(const EmuPlan& e, const Problem& p, const Tables<double>&
                  (long long)p.d.G * p.d.Nt * p.d.Np * ((p.d.NT * p.d.NP + 127) / 128)};
   return e.gRad.threads == 256 ? launch_rad_mode<256>(e, p, t, A, s)
                                : launch_rad_mode<512>(e, p, t, A, s);
+}
+
+cudaError_t emu_radial_T(const EmuPlan& e, const Problem& p, const Tables<double>& t,
+                         const double* X, double scale, bool tau, double* lt, double* Ubar,
+                         cudaStream_t s) {
+  emu::RadArgs A{X, nullptr, 1.0, tau ? 1 : 0, emu::RAD_ADJOINT, nullptr, lt, nullptr, Ubar, scale,
+                 (long long)p.d.G * p.d.Nt * p.d.Np * ((p.d.NT * p.d.NP + 127) / 128)};
+  return e.gRad.threads == 256
+             ? launch_rad<256, emu::RAD_ADJOINT>(e.gRad, e.radTM, p, t, A, s)
+             : launch_rad<512, emu::RAD_ADJOINT>(e.gRad, e.radTM, p, t, A, s);
 }
 
 }  // namespace ts

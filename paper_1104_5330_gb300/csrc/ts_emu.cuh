@@ -320,13 +320,21 @@ __device__ __forceinline__ void copy_in(unsigned char* dst, const void* src, int
 // The Fourier results (and, in the angular pass, the Phi sums that make up the
 // scattering moments) go through shared memory to the threads that finish the
 // points from the DFS results.
-enum EmuPass { EP_ANGULAR = 0, EP_PLANE = 1 };
+// EP_ADJOINT is the transposed angular pass: the same contractions with the transposed
+// matrices, lt in place of U, and the adjoint's own epilogue.
+enum EmuPass { EP_ANGULAR = 0, EP_PLANE = 1, EP_ADJOINT = 2 };
 
 struct EmuArgs {
   const double* U;
   double* K;
   double sgn;
   int collision, cons;
+  // EP_ADJOINT: K holds Ubar (read); gradients, adjoint fields and their weights
+  const double* Us;
+  double *gk, *ge;
+  const double *lam, *lam_in;
+  double *lam_out, *Kbar;
+  double wl, wu;
   int vec;   // plane: four columns start on 32 bytes and lie in one half circle
   long long ntiles;
 };
@@ -364,7 +372,7 @@ struct TileAt {
 template <int PASS>
 __device__ __forceinline__ TileAt<PASS> tile_at(const Dims& d, long long tile) {
   TileAt<PASS> r;
-  if (PASS == EP_ANGULAR) {
+  if (PASS != EP_PLANE) {
     r.b0 = tile * 8;
   } else {
     const unsigned nch = (unsigned)(d.NP / 2 + 3) / 4u;
@@ -389,7 +397,7 @@ __device__ __forceinline__ void load_units(const Dims& d, const double* F, const
 #pragma unroll
     for (int x = 0; x < 8; ++x) v[q][x] = 0.0;
     if (ua[q] < 0) continue;
-    if (PASS == EP_ANGULAR) {
+    if (PASS != EP_PLANE) {
       const double* src = F + at.b0 * S + ua[q] * Nb + ub[q];
 #pragma unroll
       for (int x = 0; x < 8; ++x)
@@ -433,6 +441,7 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
   unsigned long long* jsum = reinterpret_cast<unsigned long long*>(xm + 80);   // [10][8]
   int64_t* wqt = reinterpret_cast<int64_t*>(jsum + 80);           // angular: weights [Na]
   int* hs = reinterpret_cast<int*>(jsum + 80);                    // plane: shifts [Na]
+  double* gp = reinterpret_cast<double*>(wqt + Na);               // adjoint: [mt1][warps][8]
   int64_t* ex = reinterpret_cast<int64_t*>(sm + g.oEx);           // [Nb][a][8 x]
 
   if (Na % 8 || Nb % 16) {   // K paddings read as zero
@@ -469,17 +478,21 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
   }
   const int row = (warp & 3) * 32 + lane, grp = warp >> 2, rx = row & 7, rg = row >> 3;
   const int jobs = g.mt2 + g.mt1, ahead = g.dual ? 2 : 1;
-  const int S = PASS == EP_ANGULAR ? Na * Nb : d.NT * d.NP, hP = d.NP / 2;
+  const int S = PASS != EP_PLANE ? Na * Nb : d.NT * d.NP, hP = d.NP / 2;
   // The combination W of the two contractions stays in fixed point: a multiply of two
-  // 64-bit integers costs about a sixth of an FP64 one here. Unit of W: 2^h times that
+  // 64-bit integers takes 28 issue slots of a warp, an FP64 one 64. Unit of W: 2^h times that
   // of the DFS results; h makes room for the Fourier term's coefficient, delta is the
   // difference of the two matrices' scales.
   const int delta = m2.se - m1.se;
+  const int lgNa = 32 - __clz(Na - 1);
   for (int a = tid; a < Na; a += T) {
     if (PASS == EP_PLANE)
       hs[a] = max(2, 3 + delta + ilogb(t.inv_sinth[a]));
     else   // weights of the moments (Fejer x trapezoid; conservative: of Fhat / sinTh)
-      wqt[a] = __double2ll_rn((A.cons ? t.qdir[a] / t.sinT[a] : t.qdir[a]) * pow2(63));
+      // (adjoint: plain sums, scaled down by the power of two that holds Na rows)
+      wqt[a] = __double2ll_rn(PASS == EP_ADJOINT ? pow2(63 - lgNa)
+                                                 : (A.cons ? t.qdir[a] / t.sinT[a] : t.qdir[a]) *
+                                                       pow2(63));
   }
   double v[U][8];
   TileAt<PASS> at{};
@@ -502,7 +515,7 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
   if ((long long)blockIdx.x < A.ntiles) {
     at = tile_at<PASS>(d, blockIdx.x);
     load_units<PASS, U>(d, A.U, at, S, hP, Nb, A.vec, ua, ub, v);
-    if (PASS == EP_ANGULAR && warp == 1 && lane < 8) scalars_load(lane, 0);
+    if (PASS != EP_PLANE && warp == 1 && lane < 8) scalars_load(lane, 0);
   }
   int coef_n = -1;   // the Fourier coefficient this thread holds, and for what
   double coef_key = 0.0;
@@ -536,10 +549,10 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
         if (lane < 8) atomicMax(&smax[buf * 8 + lane], mine);
       }
     }
-    if (PASS == EP_ANGULAR && warp == 1) cp8_wait();   // this tile's scalars
+    if (PASS != EP_PLANE && warp == 1) cp8_wait();   // this tile's scalars
     __syncthreads();   // the maxima and scalars; the previous tile is finished
     if (tid < 8) smax[(buf ^ 1) * 8 + tid] = 0;
-    if (PASS == EP_ANGULAR && tid < 80) jsum[tid] = 0;
+    if (PASS != EP_PLANE && tid < 80) jsum[tid] = 0;
     // ---- digits
     {
       uint32_t em[8];
@@ -638,6 +651,7 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
     const int eb = block_exp(smax[buf * 8 + (PASS == EP_PLANE ? 0 : rx)]);
     const double* xc = xs + buf * 64;   // the scalars of this tile
     for (int n = 0; n < jobs; ++n) {
+      double gks = 0.0;   // adjoint: this thread's share of sum lt Us
       for (const int upto = min(n + ahead, jobs); issued < upto; ++issued)
         if (uwarp == T / 32 - 1) issue(issued);
       if (n == 0) {
@@ -645,7 +659,7 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
         if (tile + gridDim.x < A.ntiles) {
           at = tile_at<PASS>(d, tile + gridDim.x);
           load_units<PASS, U>(d, A.U, at, S, hP, Nb, A.vec, ua, ub, v);
-          if (PASS == EP_ANGULAR && warp == 1 && lane < 8) scalars_load(lane, buf ^ 1);
+          if (PASS != EP_PLANE && warp == 1 && lane < 8) scalars_load(lane, buf ^ 1);
         }
       }
       if (n < g.mt2) {
@@ -654,13 +668,13 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
       const bool val = a < Na;
       // the row's coefficient: sinTh cot th (angular), sinPh / sin th (plane). The
       // CTA's next tile mostly has the same th or Phi columns: kept while it does
-      const double key = PASS == EP_ANGULAR ? xc[16 + rx] : (double)cur.m0;
+      const double key = PASS != EP_PLANE ? xc[16 + rx] : (double)cur.m0;
       if (n != coef_n || key != coef_key) {
         coef_n = n;
         coef_key = key;
         coef = ws = wc = 0;
         if (val) {
-          if (PASS == EP_ANGULAR) {
+          if (PASS != EP_PLANE) {
             const double st = t.sinT[a], ct = t.cosT[a];
             coef = __double2ll_rn(st * key * pow2(64 + delta - cot_shift(key, delta)));
             if (KF >= KF_LINEAR) {
@@ -676,7 +690,7 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
       }
       wait_job(n);
       const uint32_t tl = lanes(n);
-      const int nreal = Nb + (PASS == EP_ANGULAR && A.collision ? g.nf - g.nz : 0);
+      const int nreal = Nb + (PASS != EP_PLANE && A.collision ? g.nf - g.nz : 0);
       int64_t* exr = ex + a * 8 + rx;
       for (int q = grp; 4 * q < nreal; q += NG) {
         uint32_t bb[8][4];
@@ -686,7 +700,7 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
         recombine4(bb, R);
         // functionals: outputs 0 and Nb/2 (whose derivative rows vanish, nz of them) and
         // those from Nb on
-        const bool special = PASS == EP_ANGULAR &&
+        const bool special = PASS != EP_PLANE &&
                              ((g.nz > 0 && q == 0) || (g.nz > 1 && q == hb / 4) || 4 * q + 4 > Nb);
         if (!special) {
           if (val) {
@@ -726,15 +740,17 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
       const int b = 16 * (n - g.mt2) + rg;
       const int w = PASS == EP_PLANE && b >= hb ? rx ^ 4 : rx;
       bool val = b < Nb;
+      long long po = 0;   // adjoint: this column's offset in the fields
       double* Kp;
       const double* Ip;   // what the epilogue reads per point: U (angular) or K (plane)
       unsigned st;        // stride of a (a plane spans less than 2^32 elements)
-      if (PASS == EP_ANGULAR) {
+      if (PASS != EP_PLANE) {
         val = val && cur.b0 + rx < d.nblk;
         const long long o = (cur.b0 + rx) * S + b;
         Kp = A.K + o;
         Ip = A.U + o;
         st = Nb;
+        po = o;
       } else {
         val = val && cur.m0 + (w & 3) < hP;
         Kp = A.K + cur.base + (long long)b * d.S_l + cur.m0 + (w & 3) + (w >= 4 ? hP : 0);
@@ -769,7 +785,7 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
         if (A.collision) {
           const double ks = xc[32 + w], J = xm[w];
           kks = xc[8 + w] + ks;
-          src = fma(ks, J, A.cons ? xm[72 + w] : xc[24 + w]);
+          src = PASS == EP_ADJOINT ? ks * J : fma(ks, J, A.cons ? xm[72 + w] : xc[24 + w]);
           if (KF >= KF_LINEAR) {
             const double cp = t.cosP[val ? b : 0], sp = t.sinP[val ? b : 0];
             const double kb = p.scb ? ks * xc[40 + w] : 0.0;
@@ -805,8 +821,8 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
             const int a = min(4 * q + e, Na - 1);
-            const int ha = PASS == EP_ANGULAR ? hx : hs[a];
-            if (PASS == EP_ANGULAR) W[e] >>= hx;
+            const int ha = PASS != EP_PLANE ? hx : hs[a];
+            if (PASS != EP_PLANE) W[e] >>= hx;
             else W[e] = __mul64hi(W[e], cth) >> (ha - 2);
             W[e] += exr[a * 8];
             qb[e] = qv + ha;
@@ -834,6 +850,18 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
                   gain = fma(ct, u1, fma(sT, u2, gain));
                 }
                 if (A.cons) gain *= t.sinT[a];
+                if (PASS == EP_ADJOINT) {
+                  if (val) {
+                    const long long gi = po + (unsigned)a * st;
+                    gks = fma(in[h][e], A.Us[gi], gks);
+                    const double ub = fma(c0, y4[e], fma(t.qdir[a], gain,
+                                                         fma(-kks, in[h][e], A.K[gi])));
+                    const double l0 = A.lam_in[gi];
+                    if (A.Kbar) A.Kbar[gi] = fma(A.wl, A.lam[gi], A.wu * ub);
+                    A.lam_out[gi] = l0 + ub;
+                  }
+                  continue;
+                }
                 col = fma(-kks, in[h][e], gain);
               }
               r2 = fma(c0, y4[e], col);
@@ -843,15 +871,27 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
         }
       }
       }
+      if (PASS == EP_ADJOINT && n >= g.mt2) {
+        gks += __shfl_xor_sync(0xFFFFFFFFu, gks, 8);
+        gks += __shfl_xor_sync(0xFFFFFFFFu, gks, 16);
+        if (lane < 8) gp[((n - g.mt2) * (T / 32) + warp) * 8 + lane] = gks;
+      }
       alive = end_job(n);
       if (!alive) break;
-      if (PASS == EP_ANGULAR && n == g.mt2 - 1 && A.collision) {
+      if (PASS == EP_ADJOINT && n == jobs - 1 && tid < 8 && cur.b0 + tid < d.nblk) {
+        double gt = 0.0;   // the warps' shares in a fixed order
+        for (int z = 0; z < g.mt1 * (T / 32); ++z) gt += gp[z * 8 + tid];
+        A.gk[cur.b0 + tid] -= gt;
+        A.ge[cur.b0 + tid] += xm[tid];
+      }
+      if (PASS != EP_PLANE && n == g.mt2 - 1 && A.collision) {
         if (tid < 80) {
       // moment z of block x as a double (visible after the next wait's barrier)
       const int z = tid >> 3, x = tid & 7;
       constexpr int nm = KF == KF_ISO ? 1 : KF == KF_LINEAR ? 4 : 9;
       if (z < nm) {
-        const int more = z == 0 ? 1 : z < 4 ? 3 : 5;   // 2 and 4 per factor, as exponents
+        // 2 and 4 per factor, as exponents (adjoint: and its weight's)
+        const int more = (z == 0 ? 1 : z < 4 ? 3 : 5) + (PASS == EP_ADJOINT ? lgNa : 0);
         const int qv = block_exp(smax[buf * 8 + x]) + m2.se + more;
         uint32_t top;
         const int64_t R = (int64_t)jsum[tid];
@@ -884,9 +924,11 @@ struct RadArgs {
   double sgn;
   int tau, mode;
   double *F, *Acc, *Uout, *out;
-  double dt;
+  double dt;   // adjoint: the scale of X
   long long ntiles;
 };
+constexpr int RAD_ADJOINT = 100;   // MODE of the transposed pass: U = X, Acc = lt, out = Ubar
+
 struct RadMats {
   const uint16_t* dev[8];
   const int* se[8];
@@ -914,6 +956,8 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
   volatile int* dead = reinterpret_cast<volatile int*>(ms + 20);   // a wait ran out
   uint32_t* smax = reinterpret_cast<uint32_t*>(ms + 24);   // [2]
   int* se = reinterpret_cast<int*>(ms + 32);               // [ng * n]
+  double* tot = reinterpret_cast<double*>(ms + 32 + (g.ng * g.n * 4 + 15) / 16 * 16);   // [128]
+  double* ts = reinterpret_cast<double*>(sm + g.oA);       // adjoint: [warps][128], before the digits
   if (!g.left || Nr != 8 * g.kc + 1) {   // K paddings read as zero
     for (int x = tid; x < g.oB / 16; x += T)
       reinterpret_cast<uint4*>(sm)[x] = make_uint4(0, 0, 0, 0);
@@ -969,8 +1013,8 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
       const int w = (u & 7) * 16;
       if (w < Wc) {
         const long long gi = base + (long long)(u >> 3) * d.S_i + w;
-        prefetch_line(A.Kin + gi);
-        if (MODE != RAD_RHS) prefetch_line(A.F + gi);
+        if (MODE != RAD_ADJOINT) prefetch_line(A.Kin + gi);
+        if (MODE != RAD_RHS && MODE != RAD_ADJOINT) prefetch_line(A.F + gi);
         if (rA) prefetch_line(A.Acc + gi);
       }
     }
@@ -1000,6 +1044,64 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
     };
 #pragma unroll
     for (int q = 0; q < U; ++q) load_unit(tid + q * T, v[q]);
+    if (MODE == RAD_ADJOINT) {
+      // lt = Tau^T (scale X): every row but the inflow one as it is, that one less
+      // T_N(x_b) sum_i T_N(x_i) X_i. The units hold all nodes (host): a thread's share
+      // of its eight columns' sums, then the half warps', then the CTA's, in fixed order
+#pragma unroll
+      for (int q = 0; q < U; ++q)
+#pragma unroll
+        for (int x = 0; x < 8; ++x) v[q][x] *= A.dt;
+      if (A.tau) {
+        double sum[8];
+#pragma unroll
+        for (int x = 0; x < 8; ++x) {
+          sum[x] = 0.0;
+#pragma unroll
+          for (int q = 0; q < U; ++q) {
+            const int i = (tid + q * T) >> 4;
+            if (i < Nr) sum[x] += (N - i) & 1 ? -v[q][x] : v[q][x];
+          }
+          sum[x] += __shfl_xor_sync(0xFFFFFFFFu, sum[x], 16);
+          if (lane < 16) ts[(warp * 16 + lane) * 8 + x] = sum[x];
+        }
+        __syncthreads();
+        if (tid < 128) {
+          double z = 0.0;
+          for (int w = 0; w < T / 32; ++w) z += ts[w * 128 + tid];
+          tot[tid] = z;
+        }
+        __syncthreads();
+        if (!g.left || Nr != 8 * g.kc + 1) {   // the K paddings under the sums are zero again
+          for (int x = tid; x < T * 2; x += T)
+            reinterpret_cast<uint4*>(ts)[x] = make_uint4(0, 0, 0, 0);
+        }
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+          const int i = (tid + q * T) >> 4, w = (tid & 15) * 8;
+          if (i != 0 && i != N) continue;
+#pragma unroll
+          for (int x = 0; x < 8; ++x)
+            if (w + x < Wc && i == (t.cosT[(c0 + w + x) / NP] > 0.0 ? 0 : N))
+              v[q][x] -= (N - i) & 1 ? -tot[w + x] : tot[w + x];
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        const int u = tid + q * T, w = (u & 15) * 8;
+        if (u >= Nr * 16) continue;
+        double* dst = A.Acc + base + (long long)(u >> 4) * d.S_i + w;
+        if (w + 8 <= Wc) {
+#pragma unroll
+          for (int x = 0; x < 8; x += 2)
+            *reinterpret_cast<double2*>(dst + x) = make_double2(v[q][x], v[q][x + 1]);
+        } else {
+#pragma unroll
+          for (int x = 0; x < 8; ++x)
+            if (w + x < Wc) dst[x] = v[q][x];
+        }
+      }
+    }
 #pragma unroll
     for (int q = 0; q < U; ++q)
 #pragma unroll
@@ -1082,8 +1184,8 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
     const double* Fc = A.F + base + row;
     const double* Ac = A.Acc + base + row;
     const unsigned Si = (unsigned)d.S_i;   // a group spans less than 2^32 elements (host)
-    double kb = val && A.tau ? Kc[(unsigned)bn * Si] : 0.0;
-    double* dst = (MODE == RAD_RHS ? A.out
+    double kb = MODE != RAD_ADJOINT && val && A.tau ? Kc[(unsigned)bn * Si] : 0.0;
+    double* dst = (MODE == RAD_RHS || MODE == RAD_ADJOINT ? A.out
                    : MODE == RAD_STAGE3 || MODE == RAD_AB2 || MODE == RAD_AB2_START ? A.F
                                                                                     : A.Uout) +
                   base + row;
@@ -1101,8 +1203,8 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
         noff[e] = (unsigned)(o < no ? rad_row(n * g.go + o, N) : 0) * Si;
         nk[e] = nf[e] = na[e] = 0.0;
         if (val && o < no) {
-          nk[e] = Kc[noff[e]];
-          if (MODE != RAD_RHS) nf[e] = Fc[noff[e]];
+          if (MODE != RAD_ADJOINT) nk[e] = Kc[noff[e]];
+          if (MODE != RAD_RHS && MODE != RAD_ADJOINT) nf[e] = Fc[noff[e]];
           if (rA) na[e] = Ac[noff[e]];
         }
       }
@@ -1127,7 +1229,7 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
       phase ^= 1u << r;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t tl = tmem + r * (uint32_t)g.half + ((uint32_t)((warp & 3) * 32) << 16);
-      if (n == 0 && A.tau) {   // the finished rate at the inflow node (both rows lead this group)
+      if (MODE != RAD_ADJOINT && n == 0 && A.tau) {   // the finished rate at the inflow node (both rows lead this group)
         uint32_t b[8][4];
         tm_ld(tl, g.n, b);
         tm_wait(b);
@@ -1170,6 +1272,10 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
           const int o = 4 * q + e;
           if (o >= no) break;
           const double y = y4[e];
+          if (MODE == RAD_ADJOINT) {   // Ubar = -cosTh D_r^T lt
+            if (val) dst[off[e]] = -cT * y;
+            continue;
+          }
           double v = fma(ck, y, kv[e]);
           if (A.tau) {   // K_i -= K_b T_N(x_b) T_N(x_i)
             const int flip = ((N - rad_row(n * g.go + o, N)) & 1) << 31;

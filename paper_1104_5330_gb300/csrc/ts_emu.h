@@ -47,10 +47,13 @@ constexpr int kEmuForms = 3;   // functionals of the isotropic, linear and quadr
 
 struct EmuPlan {
   void* mem = nullptr;       // every table of the plan
-  bool ang = false, plane = false, rad = false;
+  bool ang = false, plane = false, rad = false;      // which passes it covers,
+  bool adj = false, planeT = false, radT = false;    // and which transposed ones
   EmuMat angD, angF[kEmuForms], plD, plF;
   EmuGeo gAng[kEmuForms], gPl;
-  EmuMat radM[8];            // one per output group
+  EmuMat adjD, adjF[kEmuForms], plTD, plTF;   // transposed operators
+  EmuGeo gAdj[kEmuForms];
+  EmuMat radM[8], radTM[8];  // one per output group
   EmuRadGeo gRad;
 };
 
@@ -67,6 +70,10 @@ inline bool emu_has_angular(const EmuPlan& e, const Dims& d) { return e.ang && e
 inline bool emu_has_plane(const EmuPlan& e, const Dims& d) { return e.plane && emu_small(d); }
 inline bool emu_has_radial(const EmuPlan& e, const Dims& d) { return e.rad && emu_small(d); }
 
+inline bool emu_has_angular_T(const EmuPlan& e, const Dims& d) { return e.adj && emu_small(d); }
+inline bool emu_has_plane_T(const EmuPlan& e, const Dims& d) { return e.planeT && emu_small(d); }
+inline bool emu_has_radial_T(const EmuPlan& e, const Dims& d) { return e.radT && emu_small(d); }
+
 cudaError_t emu_angular(const EmuPlan& e, const Problem& p, const Tables<double>& t, bool cons,
                         const double* U, double* K, double sgn, bool collision, cudaStream_t s);
 cudaError_t emu_plane(const EmuPlan& e, const Problem& p, const Tables<double>& t,
@@ -74,5 +81,15 @@ cudaError_t emu_plane(const EmuPlan& e, const Problem& p, const Tables<double>& 
 cudaError_t emu_radial(const EmuPlan& e, const Problem& p, const Tables<double>& t,
                        const double* U, const double* K, double sgn, bool tau, int mode, double* F,
                        double* Acc, double* Uout, double* out, double dt, cudaStream_t s);
+// The transposed passes (see Launch::radial_T, plane_T, angular_T).
+cudaError_t emu_radial_T(const EmuPlan& e, const Problem& p, const Tables<double>& t,
+                         const double* X, double scale, bool tau, double* lt, double* Ubar,
+                         cudaStream_t s);
+cudaError_t emu_plane_T(const EmuPlan& e, const Problem& p, const Tables<double>& t,
+                        const double* lt, double* Ubar, cudaStream_t s);
+cudaError_t emu_angular_T(const EmuPlan& e, const Problem& p, const Tables<double>& t,
+                          const double* lt, const double* Ubar, const double* Us, double* gk,
+                          double* ge, const double* lam, const double* lam_in, double* lam_out,
+                          double* Kbar, double wl, double wu, cudaStream_t s);
 
 }  // namespace ts

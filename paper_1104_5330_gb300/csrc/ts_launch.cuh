@@ -314,6 +314,10 @@ cudaError_t Launch<T, C>::radial(const Problem& p, const Tables<C>& t, const dou
 template <typename T, typename C>
 cudaError_t Launch<T, C>::radial_T(const Problem& p, const Tables<C>& t, const T* X,
                                    double scale, bool tau, T* lt, T* Ubar, cudaStream_t s) {
+  if constexpr (sizeof(T) == 8) {
+    if (p.emu && emu_has_radial_T(*p.emu, p.d))
+      return emu_radial_T(*p.emu, p, t, X, scale, tau, lt, Ubar, s);
+  }
   static bool init = false;
   if (!init) {
     const cudaError_t ea = allow_smem(k_radial_T<T, C>);
@@ -333,6 +337,9 @@ cudaError_t Launch<T, C>::radial_T(const Problem& p, const Tables<C>& t, const T
 template <typename T, typename C>
 cudaError_t Launch<T, C>::plane_T(const Problem& p, const Tables<C>& t, const T* lt, T* Ubar,
                                   cudaStream_t s) {
+  if constexpr (sizeof(T) == 8) {
+    if (p.emu && emu_has_plane_T(*p.emu, p.d)) return emu_plane_T(*p.emu, p, t, lt, Ubar, s);
+  }
   static bool init = false;
   if (!init) {
     cudaError_t ea = allow_smem(k_plane_T<T, C>);
@@ -357,6 +364,11 @@ cudaError_t Launch<T, C>::angular_T(const Problem& p, const Tables<C>& t, const 
                                     const T* Ubar, const T* Us, double* gk, double* ge,
                                     const T* lam, const T* lam_in, T* lam_out, T* Kbar_out,
                                     double wl, double wu, cudaStream_t s) {
+  if constexpr (sizeof(T) == 8) {
+    if (p.emu && emu_has_angular_T(*p.emu, p.d))
+      return emu_angular_T(*p.emu, p, t, lt, Ubar, Us, gk, ge, lam, lam_in, lam_out, Kbar_out, wl,
+                           wu, s);
+  }
   static bool init = false;
   if (!init) {
     const cudaError_t ea = allow_smem(k_angular_T<T, C>);

@@ -148,3 +148,32 @@ def test_a_wait_that_runs_out_is_reported_and_the_grid_recovers():
     ts.ts_sync_status(gg.handle)
     ts.ts_set_wait_limit(gg.handle, 0)
     assert rel_l2(host(_rhs(gg, cuda(F0))), op.rhs(F0)) < 1e-12
+
+
+@pytest.mark.parametrize("form", ["iso", "linear", "thomson"])
+@pytest.mark.parametrize("n", SHAPES[2:], ids=str)
+def test_adjoint_step_matches_the_oracle(n, form):
+    if form != "iso" and min(n[3], n[4]) < 4:
+        pytest.skip("the anisotropic kernels need more directions")
+    dims = (0.2, 1.0) + n
+    og, gg = pair(*dims, G=2)
+    kap, eta, ks, F0, g1, g2 = absorber_workload(og)
+    kw = {}
+    if form == "linear":
+        gg.set_scattering_anisotropy(-0.3)
+        kw = dict(scatter_b=-0.3)
+    elif form == "thomson":
+        gg.set_scattering_quadrupole(0.75)
+        kw = dict(scatter_c=0.75)
+    gg.set_coeffs(kap, eta, ks, g1, g2)
+    op = OProblem(og, kap, eta, ks, g1, g2, **kw)
+    dt = 0.05 / (n[0] ** 2 + 4 * n[1] * n[2] + n[3] * n[4] * n[1])
+    lam0 = np.random.default_rng(5).standard_normal(og.shape)
+    lam = cuda(lam0)
+    gk = torch.zeros(gg.coef_shape, dtype=torch.float64, device="cuda")
+    ge = torch.zeros_like(gk)
+    gg.adjoint_step(cuda(F0), lam, gk, ge, dt)
+    T().ts_sync_status(gg.handle)
+    lo, gko, geo = op.adjoint_step(F0, lam0, dt)
+    for a, b in ((lam, lo), (gk, gko), (ge, geo)):
+        assert rel_l2(host(a), b) < 1e-12

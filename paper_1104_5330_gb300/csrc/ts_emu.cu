@@ -186,8 +186,11 @@ int region(int n) { return 8 * n + (n % 16 ? 16 : 0); }
 constexpr int kTwoCtas = 113 * 1024;   // shared memory of each of two CTAs on an SM
 constexpr int kOneCta = 227 * 1024;
 
-bool geometry2(int Na, int Nb, const EmuMat& D, const EmuMat& F, int nf, int nz, EmuGeo* out) {
+bool geometry2_form(int xw, bool seq, int Na, int Nb, const EmuMat& D, const EmuMat& F, int nf,
+                    int nz, EmuGeo* out) {
   EmuGeo g{};
+  g.xw = xw;
+  g.seq = seq ? 1 : 0;
   g.Na = Na;
   g.Nb = Nb;
   g.hb = Nb / 2;
@@ -201,37 +204,39 @@ bool geometry2(int Na, int Nb, const EmuMat& D, const EmuMat& F, int nf, int nz,
   g.n2 = F.n;
   g.r1 = D.rows;
   g.r2 = F.rows;
-  g.mt1 = (Nb + 15) / 16;
-  g.mt2 = (Na + 15) / 16;
-  // copy 1: 16 bytes more per row group, so that the stores of a warp (consecutive b)
-  // fall on distinct banks
-  g.sb1 = g.ka * 128 + 16;
-  g.d1 = (Nb + g.hb) * g.sb1;
+  g.mt1 = (Nb * xw + 127) / 128;
+  g.mt2 = (Na * xw + 127) / 128;
+  const int hg = g.hb * xw / 8;   // row groups of half the Fourier axis
+  // copy 1: 16 (32) bytes more per row group, so that the stores of a warp (consecutive
+  // b; or pairs of a) fall on distinct banks
+  g.sb1 = g.ka * 128 + (xw == 8 ? 16 : 32);
+  g.d1 = 3 * hg * g.sb1;
   g.sb2 = g.kb * 128;
-  g.d2 = Na * g.sb2;
-  g.exP = Na * 8 + 8;
+  g.d2 = (Na * xw + 7) / 8 * g.sb2;
+  g.exP = Na * xw + 8;
   const int exB = Nb * g.exP * 8;
-  const bool alias = g.mt2 == 1 && Na % 8 == 0 && Nb % 8 == 0 && exB <= 8 * g.d2;
+  const bool alias =
+      xw == 8 && g.mt2 == 1 && Na % 8 == 0 && Nb % 8 == 0 && exB <= 8 * g.d2;
   int o = 0;
   auto take = [&](int bytes) {
     const int at = o;
     o += (bytes + 127) / 128 * 128;
     return at;
   };
-  g.oC1 = take(8 * g.d1);
-  g.oC2 = take(8 * g.d2);
+  g.oC1 = take(seq ? 8 * std::max(g.d1, g.d2) : 8 * g.d1);
+  g.oC2 = seq ? g.oC1 : take(8 * g.d2);
   g.oB1 = take(D.bytes());
   g.oB2 = take(F.bytes());
   g.oCA = take(2 * 128 * 16);
   g.oEx = alias ? g.oC2 : take(exB);
   g.oMs = take(96 + (128 + 160 + Na + g.mt1 * 16 * 8) * 8);
   // a 128-row tile may read row groups past the last one: inside the allocation
-  const int over = std::max(g.oC1 + 7 * g.d1 + (16 * g.mt1 + g.hb) * g.sb1 + 256,
+  const int over = std::max(g.oC1 + 7 * g.d1 + (16 * g.mt1 + hg) * g.sb1 + 256,
                             g.oC2 + 7 * g.d2 + 16 * g.mt2 * g.sb2 + 256);
   g.bytes = (std::max(o, over) + 127) / 128 * 128;
   const int reg = std::max(region(g.n1), region(g.n2));
   if (reg > 512 || Na * Nb > 1024) return false;
-  if (g.bytes <= kTwoCtas && reg <= 256 && Na * Nb <= 512) {
+  if (xw == 8 && g.bytes <= kTwoCtas && reg <= 256 && Na * Nb <= 512) {
     g.threads = 256;
     g.half = pow2_at_least(reg);
     g.dual = g.half <= 128 && (g.mt2 == 1 || !alias);
@@ -244,8 +249,18 @@ bool geometry2(int Na, int Nb, const EmuMat& D, const EmuMat& F, int nf, int nz,
   } else {
     return false;
   }
+  if (xw == 4 && (Na + 1) / 2 * Nb > g.threads) return false;   // one unit a thread
+  if (seq && g.mt2 > (g.dual ? 2 : 1)) return false;
   *out = g;
   return true;
+}
+// Eight x where both copies fit; else four (which need whole pairs in each half of the
+// Fourier axis), with the copies in one buffer if need be.
+bool geometry2(int Na, int Nb, const EmuMat& D, const EmuMat& F, int nf, int nz, EmuGeo* out) {
+  if (geometry2_form(8, false, Na, Nb, D, F, nf, nz, out)) return true;
+  if (Nb % 4) return false;
+  return geometry2_form(4, false, Na, Nb, D, F, nf, nz, out) ||
+         geometry2_form(4, true, Na, Nb, D, F, nf, nz, out);
 }
 
 bool geometry_radial(int Nr, EmuRadGeo* out) {
@@ -255,11 +270,15 @@ bool geometry_radial(int Nr, EmuRadGeo* out) {
   g.kc = g.left ? (Nr - 1) / 8 : (Nr + 15) / 16 * 2;
   g.sb = g.kc * 128 + 16;
   g.d = 16 * g.sb;
-  for (int two = 1; two >= 0; --two) {
+  // two CTAs on an SM; one; one with the matrices streamed through two buffers
+  for (int form = 0; form < 3; ++form) {
+    const bool two = form == 0;
     for (int go = 32; go >= 8; go -= 8) {   // outputs per group: whole cores, fewest groups
       const int ng = (Nr + go - 1) / go;
       if (ng > 8) break;
       g.ng = ng;
+      g.nb = form == 2 ? 2 : ng;
+      if (form == 2 && ng < 3) continue;
       g.go = (Nr + ng - 1) / ng;
       g.n = (g.go + 7) / 8 * 8;
       g.rows = 8 * g.n + 16;
@@ -273,15 +292,16 @@ bool geometry_radial(int Nr, EmuRadGeo* out) {
         return at;
       };
       g.oA = take(8 * g.d + 256);
-      g.oB = take(ng * g.bB);
+      g.oB = take(g.nb * g.bB);
       g.oCA = take(2 * 128 * 16);
-      g.oMs = take(32 + (ng * g.n * 4 + 15) / 16 * 16 + 128 * 8);
+      g.oMs = take(64 + (ng * g.n * 4 + 15) / 16 * 16 + 128 * 8);
       g.bytes = o;
       if (g.bytes > (two ? kTwoCtas : kOneCta)) continue;
       g.threads = two ? 256 : 512;
       g.half = pow2_at_least(reg);
       g.dual = g.half <= (two ? 128 : 256) && ng > 1;
       g.cols = g.dual ? 2 * g.half : g.half;
+      if (form == 2 && !g.dual) continue;
       *out = g;
       return true;
     }
@@ -487,15 +507,15 @@ cudaError_t emu_ctas(int threads, long long ntiles, int* ctas) {
   return e;
 }
 
-template <int PASS, int KF, int T, int U, int NA, int NB>
+template <int PASS, int KF, int T, int U, int NA, int NB, int XW = 8>
 cudaError_t launch2(const Problem& p, const Tables<double>& t, const EmuGeo& g, const EmuMat& D,
                     const EmuMat& F, emu::EmuArgs A, cudaStream_t s) {
-  static const cudaError_t e = allow_smem(emu::k_emu2<PASS, KF, T, U, NA, NB>);   // once per kernel
+  static const cudaError_t e = allow_smem(emu::k_emu2<PASS, KF, T, U, NA, NB, XW>);   // once per kernel
   if (e != cudaSuccess) return e;
   int ctas = 1;
   const cudaError_t e2 = emu_ctas(T, A.ntiles, &ctas);
   if (e2 != cudaSuccess) return e2;
-  emu::k_emu2<PASS, KF, T, U, NA, NB><<<ctas, T, g.bytes, s>>>(p, t, g, {D.dev, 3 - D.s}, {F.dev, 3 - F.s},
+  emu::k_emu2<PASS, KF, T, U, NA, NB, XW><<<ctas, T, g.bytes, s>>>(p, t, g, {D.dev, 3 - D.s}, {F.dev, 3 - F.s},
                                                        A);
   return cudaGetLastError();
 }
@@ -504,9 +524,19 @@ template <int PASS, int KF>
 cudaError_t launch2t(const Problem& p, const Tables<double>& t, const EmuGeo& g, const EmuMat& D,
                      const EmuMat& F, emu::EmuArgs A, cudaStream_t s) {
   const bool one = g.Na * g.Nb <= g.threads;
+  const int h = g.xw / 2;
+  const uintptr_t at = reinterpret_cast<uintptr_t>(A.U);
+  if (PASS == emu::EP_PLANE) {   // h columns of a half circle in one load
+    A.ntiles = (long long)p.d.G * p.d.Nr * p.d.NT * ((p.d.NP / 2 + h - 1) / h);
+    A.vec = p.d.NP % (2 * h) == 0 && at % (8 * h) == 0;
+  } else {                       // xw = 4: two points of a row (rows are of even length)
+    A.ntiles = (p.d.nblk + g.xw - 1) / g.xw;
+    A.vec = at % 16 == 0;
+  }
   // 16 x 16, the size of most grids, has its own form: the index arithmetic folds away
   if (g.threads == 256 && g.Na == 16 && g.Nb == 16)
     return launch2<PASS, KF, 256, 1, 16, 16>(p, t, g, D, F, A, s);
+  if (g.xw == 4) return launch2<PASS, KF, 512, 1, 0, 0, 4>(p, t, g, D, F, A, s);
   if (g.threads == 256)
     return one ? launch2<PASS, KF, 256, 1, 0, 0>(p, t, g, D, F, A, s)
                : launch2<PASS, KF, 256, 2, 0, 0>(p, t, g, D, F, A, s);
@@ -525,7 +555,6 @@ cudaError_t emu_angular(const EmuPlan& e, const Problem& p, const Tables<double>
   A.sgn = sgn;
   A.collision = collision ? 1 : 0;
   A.cons = cons ? 1 : 0;
-  A.ntiles = (p.d.nblk + 7) / 8;
   switch (kf) {
     case KF_QUADRATIC:
       return launch2t<emu::EP_ANGULAR, KF_QUADRATIC>(p, t, e.gAng[kf], e.angD, e.angF[kf], A, s);
@@ -544,8 +573,6 @@ cudaError_t plane_launch(const Problem& p, const Tables<double>& t, const EmuGeo
   A.U = U;
   A.K = K;
   A.sgn = sgn;
-  A.vec = p.d.NP % 8 == 0 && (reinterpret_cast<uintptr_t>(U) & 31u) == 0;
-  A.ntiles = (long long)p.d.G * p.d.Nr * p.d.NT * ((p.d.NP / 2 + 3) / 4);
   return launch2t<emu::EP_PLANE, KF_ISO>(p, t, g, D, F, A, s);
 }
 }  // namespace
@@ -574,7 +601,6 @@ cudaError_t emu_angular_T(const EmuPlan& e, const Problem& p, const Tables<doubl
   A.Kbar = Kbar;
   A.wl = wl;
   A.wu = wu;
-  A.ntiles = (p.d.nblk + 7) / 8;
   switch (kf) {
     case KF_QUADRATIC:
       return launch2t<emu::EP_ADJOINT, KF_QUADRATIC>(p, t, e.gAdj[kf], e.adjD, e.adjF[kf], A, s);

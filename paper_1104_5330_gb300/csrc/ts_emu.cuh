@@ -307,16 +307,20 @@ __device__ __forceinline__ void copy_in(unsigned char* dst, const void* src, int
 }
 
 // ============================================================================
-// Two-axis passes. A tile is Na x Nb x 8 points (a, b, x):
-//  * angular: a = Theta, b = Phi, x = eight angular blocks;
-//  * plane: a = theta, b = phi, x = eight Phi columns, four of each half circle.
+// Two-axis passes. A tile is Na x Nb x XW points (a, b, x), XW = 8 or 4:
+//  * angular: a = Theta, b = Phi, x = XW angular blocks;
+//  * plane: a = theta, b = phi, x = XW Phi columns, half of them of each half circle.
 // The a axis is a double-Fourier-sphere axis: its operator takes the line and the
 // line of the partner (b + Nb/2; in the plane pass also the column of the other
 // half circle). The b axis is periodic. Both contractions read the tile's digits
-// as MN-major operands, rows (b, x) or (a, x) in groups of 8 x:
-//   copy 1 [digit][b in 0..Nb-1, 0..Nb/2-1][a][8 x]   -- K along a; the partner's
-//           rows start Nb/2 groups further on, hence the repeated first half;
-//   copy 2 [digit][a][b][8 x]                          -- K along b.
+// as MN-major operands, rows (b, x) or (a, x) in groups of eight (8 x of one b or a,
+// or 4 x of two):
+//   copy 1 [digit][b in 0..Nb-1, 0..Nb/2-1][a][8 rows] -- K along a; the partner's
+//           rows start Nb/2 further on, hence the repeated first half;
+//   copy 2 [digit][a][b][8 rows]                       -- K along b.
+// Where both do not fit, the tile has four x and the copies take turns in one buffer
+// (seq): copy 1 is written when the Fourier products are done; the DFS products run
+// under the Fourier epilogue.
 // The Fourier results (and, in the angular pass, the Phi sums that make up the
 // scattering moments) go through shared memory to the threads that finish the
 // points from the DFS results.
@@ -335,7 +339,7 @@ struct EmuArgs {
   const double *lam, *lam_in;
   double *lam_out, *Kbar;
   double wl, wu;
-  int vec;   // plane: four columns start on 32 bytes and lie in one half circle
+  int vec;   // the values may be loaded four (two) at a time
   long long ntiles;
 };
 
@@ -344,11 +348,13 @@ struct MatArg {
   int se;          // 3 - s of the whole matrix
 };
 
-// Adds w, summed over the warp's rows of the same x (lanes 8 apart), to a shared sum.
+// Adds w, summed over the warp's rows of the same x (lanes XW apart), to a shared sum.
+template <int XW>
 __device__ __forceinline__ void moment(unsigned long long* s, int64_t w) {
+  if (XW == 4) w += __shfl_xor_sync(0xFFFFFFFFu, w, 4);
   w += __shfl_xor_sync(0xFFFFFFFFu, w, 8);
   w += __shfl_xor_sync(0xFFFFFFFFu, w, 16);
-  if ((threadIdx.x & 31) < 8) atomicAdd(s, (unsigned long long)w);
+  if ((threadIdx.x & 31) < XW) atomicAdd(s, (unsigned long long)w);
 }
 // The shift that makes room for the coefficient sinTh cot th.
 __device__ __forceinline__ int cot_shift(double cot, int delta) {
@@ -369,15 +375,16 @@ struct TileAt {
   long long b0 = 0, base = 0;   // angular: first block; plane: (g, i, Theta) offset
   int k = 0, i = 0, m0 = 0;
 };
-template <int PASS>
+template <int PASS, int XW>
 __device__ __forceinline__ TileAt<PASS> tile_at(const Dims& d, long long tile) {
   TileAt<PASS> r;
   if (PASS != EP_PLANE) {
-    r.b0 = tile * 8;
+    r.b0 = tile * XW;
   } else {
-    const unsigned nch = (unsigned)(d.NP / 2 + 3) / 4u;
+    constexpr unsigned H = XW / 2;
+    const unsigned nch = ((unsigned)(d.NP / 2) + H - 1) / H;
     unsigned q = (unsigned)tile;   // tiles of a field fit 32 bits (checked on the host)
-    r.m0 = (int)(q % nch) * 4;
+    r.m0 = (int)(q % nch * H);
     q /= nch;
     r.k = (int)(q % (unsigned)d.NT);
     q /= (unsigned)d.NT;
@@ -387,8 +394,14 @@ __device__ __forceinline__ TileAt<PASS> tile_at(const Dims& d, long long tile) {
   }
   return r;
 }
-// The values of this thread's units (zero outside the tile).
-template <int PASS, int U>
+__device__ __forceinline__ void ld2(const double* p, double& a, double& b) {
+  const double2 y = *reinterpret_cast<const double2*>(p);
+  a = y.x;
+  b = y.y;
+}
+// The values of this thread's units (zero outside the tile). A unit is eight rows of
+// copy 1 at one a: (b; 8 x), or (b, b + 1; 4 x).
+template <int PASS, int U, int XW>
 __device__ __forceinline__ void load_units(const Dims& d, const double* F, const TileAt<PASS>& at,
                                            int S, int hP, int Nb, bool vec, const int (&ua)[U],
                                            const int (&ub)[U], double (&v)[U][8]) {
@@ -399,28 +412,54 @@ __device__ __forceinline__ void load_units(const Dims& d, const double* F, const
     if (ua[q] < 0) continue;
     if (PASS != EP_PLANE) {
       const double* src = F + at.b0 * S + ua[q] * Nb + ub[q];
-#pragma unroll
-      for (int x = 0; x < 8; ++x)
-        if (at.b0 + x < d.nblk) v[q][x] = src[x * S];
-    } else {
-      const double* src = F + at.base + (long long)ua[q] * d.S_j + (long long)ub[q] * d.S_l + at.m0;
-      if (vec) {   // four columns of a half circle at once: every lane reads its own line
-#pragma unroll
-        for (int x = 0; x < 8; x += 4)
-          asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
-                       : "=d"(v[q][x]), "=d"(v[q][x + 1]), "=d"(v[q][x + 2]), "=d"(v[q][x + 3])
-                       : "l"(src + (x ? hP : 0)));
-      } else {
+      if (XW == 8) {
 #pragma unroll
         for (int x = 0; x < 8; ++x)
-          if (at.m0 + (x & 3) < hP) v[q][x] = src[(x & 3) + (x >= 4 ? hP : 0)];
+          if (at.b0 + x < d.nblk) v[q][x] = src[x * S];
+      } else {
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+          if (at.b0 + x >= d.nblk) continue;
+          if (vec) {
+            ld2(src + x * S, v[q][x], v[q][x + 4]);
+          } else {
+            v[q][x] = src[x * S];
+            v[q][x + 4] = src[x * S + 1];
+          }
+        }
+      }
+    } else {
+      const double* src = F + at.base + (long long)ua[q] * d.S_j + (long long)ub[q] * d.S_l + at.m0;
+      if (XW == 8) {
+        if (vec) {   // four columns of a half circle at once: every lane reads its own line
+#pragma unroll
+          for (int x = 0; x < 8; x += 4)
+            asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
+                         : "=d"(v[q][x]), "=d"(v[q][x + 1]), "=d"(v[q][x + 2]), "=d"(v[q][x + 3])
+                         : "l"(src + (x ? hP : 0)));
+        } else {
+#pragma unroll
+          for (int x = 0; x < 8; ++x)
+            if (at.m0 + (x & 3) < hP) v[q][x] = src[(x & 3) + (x >= 4 ? hP : 0)];
+        }
+      } else {
+#pragma unroll
+        for (int x = 0; x < 8; x += 2) {   // pairs of columns: (b, half)
+          const double* z = src + (x >= 4 ? d.S_l : 0) + (x & 2 ? hP : 0);
+          if (vec) {
+            ld2(z, v[q][x], v[q][x + 1]);
+          } else {
+            if (at.m0 < hP) v[q][x] = z[0];
+            if (at.m0 + 1 < hP) v[q][x + 1] = z[1];
+          }
+        }
       }
     }
   }
 }
 
 // NA_, NB_: the axes' lengths at compile time (0: from the geometry).
-template <int PASS, int KF, int T, int U, int NA_, int NB_>
+template <int PASS, int KF, int T, int U, int NA_, int NB_, int XW>
 __global__ void __launch_bounds__(T, T == 256 ? 2 : 1)
 k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
   extern __shared__ __align__(128) unsigned char sm[];
@@ -429,7 +468,7 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int uwarp = __shfl_sync(0xFFFFFFFFu, warp, 0);   // warp-uniform
   constexpr int NG = T / 128;                     // threads per tensor-memory lane
-  const int Na = NA_ ? NA_ : g.Na, Nb = NB_ ? NB_ : g.Nb, hb = Nb / 2, exP = Na * 8 + 8;
+  const int Na = NA_ ? NA_ : g.Na, Nb = NB_ ? NB_ : g.Nb, hb = Nb / 2, exP = Na * XW + 8;
   // small arrays
   unsigned char* ms = sm + g.oMs;
   uint64_t* bar = reinterpret_cast<uint64_t*>(ms);
@@ -442,9 +481,9 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
   int64_t* wqt = reinterpret_cast<int64_t*>(jsum + 80);           // angular: weights [Na]
   int* hs = reinterpret_cast<int*>(jsum + 80);                    // plane: shifts [Na]
   double* gp = reinterpret_cast<double*>(wqt + Na);               // adjoint: [mt1][warps][8]
-  int64_t* ex = reinterpret_cast<int64_t*>(sm + g.oEx);           // [Nb][a][8 x]
+  int64_t* ex = reinterpret_cast<int64_t*>(sm + g.oEx);           // [Nb][a][XW]
 
-  if (Na % 8 || Nb % 16) {   // K paddings read as zero
+  if (Na % 8 || Nb % 16 || g.seq) {   // K paddings hold finite digits (their products vanish)
     for (int x = tid; x < g.oB1 / 16; x += T)
       reinterpret_cast<uint4*>(sm)[x] = make_uint4(0, 0, 0, 0);
   }
@@ -473,10 +512,18 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
 #pragma unroll
   for (int q = 0; q < U; ++q) {
     const int u = tid + q * T;
-    ua[q] = u < Na * Nb ? u / Nb : -1;
-    ub[q] = u - (u / Nb) * Nb;
+    if (XW == 8) {
+      ua[q] = u < Na * Nb ? u / Nb : -1;
+      ub[q] = u - (u / Nb) * Nb;
+    } else {   // neighbouring lanes hold a and a + 1: their halves of a row of copy 2
+      ua[q] = u / Nb * 2 + (u & 1);
+      ub[q] = (u - u / Nb * Nb) / 2 * 2;
+      if (ua[q] >= Na) ua[q] = -1;
+    }
   }
-  const int row = (warp & 3) * 32 + lane, grp = warp >> 2, rx = row & 7, rg = row >> 3;
+  const int row = (warp & 3) * 32 + lane, grp = warp >> 2, rx = row & (XW - 1), rg = row / XW;
+  constexpr int XH = XW / 2;
+  constexpr int RT = 128 / XW;                    // a's or b's of a 128-row tile
   const int jobs = g.mt2 + g.mt1, ahead = g.dual ? 2 : 1;
   const int S = PASS != EP_PLANE ? Na * Nb : d.NT * d.NP, hP = d.NP / 2;
   // The combination W of the two contractions stays in fixed point: a multiply of two
@@ -513,9 +560,9 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
     cp8(x + 448, t.sin_th + jj);
   };
   if ((long long)blockIdx.x < A.ntiles) {
-    at = tile_at<PASS>(d, blockIdx.x);
-    load_units<PASS, U>(d, A.U, at, S, hP, Nb, A.vec, ua, ub, v);
-    if (PASS != EP_PLANE && warp == 1 && lane < 8) scalars_load(lane, 0);
+    at = tile_at<PASS, XW>(d, blockIdx.x);
+    load_units<PASS, U, XW>(d, A.U, at, S, hP, Nb, A.vec, ua, ub, v);
+    if (PASS != EP_PLANE && warp == 1 && lane < XW) scalars_load(lane, 0);
   }
   int coef_n = -1;   // the Fourier coefficient this thread holds, and for what
   double coef_key = 0.0;
@@ -541,12 +588,16 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
         if (lane == 0) atomicMax(&smax[buf * 8], r);
       } else {
         uint32_t mine = 0;
+        if (XW == 4) {
 #pragma unroll
-        for (int x = 0; x < 8; ++x) {
+          for (int x = 0; x < 4; ++x) mx[x] = max(mx[x], mx[x + 4]);
+        }
+#pragma unroll
+        for (int x = 0; x < XW; ++x) {
           const uint32_t r = __reduce_max_sync(0xFFFFFFFFu, mx[x]);
           if (lane == x) mine = r;
         }
-        if (lane < 8) atomicMax(&smax[buf * 8 + lane], mine);
+        if (lane < XW) atomicMax(&smax[buf * 8 + lane], mine);
       }
     }
     if (PASS != EP_PLANE && warp == 1) cp8_wait();   // this tile's scalars
@@ -554,40 +605,67 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
     if (tid < 8) smax[(buf ^ 1) * 8 + tid] = 0;
     if (PASS != EP_PLANE && tid < 80) jsum[tid] = 0;
     // ---- digits
-    {
-      uint32_t em[8];
+    auto fence_digits = [&]() {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncthreads();
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    };
+    uint64_t f4[XW == 4 ? U : 1][8];   // kept for the second copy
+    // the copies of a unit's digits
+    auto put = [&](const uint64_t (&f)[8], int q, bool one, bool two) {
+      constexpr int H = XW / 2;
+      unsigned char* c1 = sm + g.oC1 + ub[q] * XW / 8 * g.sb1 + ua[q] * 16;
+      unsigned char* c2 = XW == 8 ? sm + g.oC2 + ua[q] * g.sb2 + ub[q] * 16
+                                  : sm + g.oC2 + (ua[q] >> 1) * g.sb2 + ub[q] * 16 + (ua[q] & 1) * 8;
+      const bool ring = ub[q] < hb, rot = PASS == EP_PLANE && !ring;
 #pragma unroll
-      for (int x = 0; x < 8; ++x)
+      for (int w = 3; w >= 0; --w) {
+        uint32_t pk[4];
+        pack_pairs(f, w, pk);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int dig = 7 - (2 * w + h);
+          const uint4 x4 = digit_of(pk, h);
+          if (two) {
+            if (XW == 8) {
+              *reinterpret_cast<uint4*>(c2 + dig * g.d2) = x4;
+            } else {
+              *reinterpret_cast<uint2*>(c2 + dig * g.d2) = make_uint2(x4.x, x4.y);
+              *reinterpret_cast<uint2*>(c2 + dig * g.d2 + 16) = make_uint2(x4.z, x4.w);
+            }
+          }
+          if (one) {   // the other half circle's columns trade places past Nb / 2
+            const uint4 y4 = !rot     ? x4
+                             : H == 4 ? make_uint4(x4.z, x4.w, x4.x, x4.y)
+                                      : make_uint4(x4.y, x4.x, x4.w, x4.z);
+            *reinterpret_cast<uint4*>(c1 + dig * g.d1) = y4;
+            if (ring) *reinterpret_cast<uint4*>(c1 + dig * g.d1 + Nb * XW / 8 * g.sb1) = y4;
+          }
+        }
+      }
+    };
+    {
+      uint32_t em[XW];
+#pragma unroll
+      for (int x = 0; x < XW; ++x)
         em[x] = fixed_key(smax[buf * 8 + (PASS == EP_PLANE ? 0 : x)]);
 #pragma unroll
       for (int q = 0; q < U; ++q) {
         if (ua[q] < 0) continue;
-        uint64_t f[8];
+        if constexpr (XW == 8) {
+          uint64_t f[8];
 #pragma unroll
-        for (int x = 0; x < 8; ++x) f[x] = to_fixed(v[q][x], em[x]);
-        unsigned char* c1 = sm + g.oC1 + ub[q] * g.sb1 + ua[q] * 16;
-        unsigned char* c2 = sm + g.oC2 + ua[q] * g.sb2 + ub[q] * 16;
-        const bool ring = ub[q] < hb, rot = PASS == EP_PLANE && !ring;
+          for (int x = 0; x < 8; ++x) f[x] = to_fixed(v[q][x], em[x]);
+          put(f, q, true, true);
+        } else {
 #pragma unroll
-        for (int w = 3; w >= 0; --w) {
-          uint32_t pk[4];
-          pack_pairs(f, w, pk);
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int dig = 7 - (2 * w + h);
-            const uint4 x4 = digit_of(pk, h);
-            *reinterpret_cast<uint4*>(c2 + dig * g.d2) = x4;
-            const uint4 y4 = rot ? make_uint4(x4.z, x4.w, x4.x, x4.y) : x4;
-            *reinterpret_cast<uint4*>(c1 + dig * g.d1) = y4;
-            if (ring) *reinterpret_cast<uint4*>(c1 + dig * g.d1 + Nb * g.sb1) = y4;
-          }
+          for (int x = 0; x < 8; ++x) f4[q][x] = to_fixed(v[q][x], em[x & 3]);
+          put(f4[q], q, !g.seq, true);
         }
       }
     }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    fence_digits();
     // issues job n (one call site: the unrolled chains are inlined there, their
     // operands in uniform registers)
     auto issue = [&](int n) {
@@ -603,7 +681,7 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
           chain_any(one, tm, ca, a, g.d2, g.sb2, g.kc2 / 2, 0, false, b, 0, g.r2, g.n2);
       } else {
         const uint32_t a = smb + g.oC1 + (uint32_t)(16 * (n - g.mt2) * g.sb1), b = smb + g.oB1;
-        const uint32_t part = (uint32_t)(hb * g.sb1);
+        const uint32_t part = (uint32_t)(hb * XW / 8 * g.sb1);
         const int ka = NA_ ? (NA_ + 7) / 8 : g.n1 <= 32 ? g.ka : 0;
         if (ka == 1)
           chain_steps<0, true, true>(one, tm, ca, a, g.d1, g.sb1, part, b, 0, g.r1, g.n1);
@@ -621,6 +699,7 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
     };
     const TileAt<PASS> cur = at;
     int issued = 0;
+    const int early = XW == 4 && g.seq ? g.mt2 : 0;   // jobs waited for ahead of their epilogue
     // waits for job n, every warp for itself; where a wait runs out the warp goes on (its
     // results are void) and all leave together after the job's barrier
     auto wait_job = [&](int n) {
@@ -638,7 +717,8 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
         // our own MMAs end before the CTA exits (full bound)
         for (int x = n; x < issued; ++x) {
           const uint32_t rr = g.dual ? (uint32_t)(x & 1) : 0u;
-          bar_wait(sm_u32(&bar[rr]), ((phase >> rr) & 1u) ^ (x == n ? 1u : 0u), kDefaultWaitIters);
+          const bool passed = x == n || x < early;   // this thread has gone past that phase
+          bar_wait(sm_u32(&bar[rr]), ((phase >> rr) & 1u) ^ (passed ? 1u : 0u), kDefaultWaitIters);
         }
         return false;
       }
@@ -652,19 +732,36 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
     const double* xc = xs + buf * 64;   // the scalars of this tile
     for (int n = 0; n < jobs; ++n) {
       double gks = 0.0;   // adjoint: this thread's share of sum lt Us
-      for (const int upto = min(n + ahead, jobs); issued < upto; ++issued)
-        if (uwarp == T / 32 - 1) issue(issued);
+      if constexpr (XW == 8) {
+        for (const int upto = min(n + ahead, jobs); issued < upto; ++issued)
+          if (uwarp == T / 32 - 1) issue(issued);
+      } else {
+#pragma unroll 1
+        for (int part = n < early ? n : 1; part < 2; ++part) {
+          for (const int upto = part ? min(n + ahead, jobs) : early; issued < upto; ++issued)
+            if (uwarp == T / 32 - 1) issue(issued);
+          if (part == 0) {   // copy 1 takes copy 2's place when the Fourier products are done
+            for (int z = 0; z < early; ++z) wait_job(z);
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < U; ++q)
+              if (ua[q] >= 0) put(f4[q], q, true, false);
+            fence_digits();
+          }
+        }
+      }
       if (n == 0) {
         // the next tile's values travel while this one is finished
         if (tile + gridDim.x < A.ntiles) {
-          at = tile_at<PASS>(d, tile + gridDim.x);
-          load_units<PASS, U>(d, A.U, at, S, hP, Nb, A.vec, ua, ub, v);
-          if (PASS != EP_PLANE && warp == 1 && lane < 8) scalars_load(lane, buf ^ 1);
+          at = tile_at<PASS, XW>(d, tile + gridDim.x);
+          load_units<PASS, U, XW>(d, A.U, at, S, hP, Nb, A.vec, ua, ub, v);
+          if (PASS != EP_PLANE && warp == 1 && lane < XW) scalars_load(lane, buf ^ 1);
         }
       }
       if (n < g.mt2) {
       // ---- Fourier results: rows (a, x), times the coefficient of their term
-      const int a = 16 * n + rg;
+      const int a = RT * n + rg;
       const bool val = a < Na;
       // the row's coefficient: sinTh cot th (angular), sinPh / sin th (plane). The
       // CTA's next tile mostly has the same th or Phi columns: kept while it does
@@ -682,16 +779,16 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
               wc = __double2ll_rn(ct * pow2(62));
             }
           } else {
-            const bool ok = cur.m0 + (rx & 3) < hP;
-            const double sp = ok ? t.sinP[cur.m0 + (rx & 3) + (rx >= 4 ? hP : 0)] : 0.0;
+            const bool ok = cur.m0 + (rx & (XH - 1)) < hP;
+            const double sp = ok ? t.sinP[cur.m0 + (rx & (XH - 1)) + (rx >= XH ? hP : 0)] : 0.0;
             coef = __double2ll_rn(sp * t.inv_sinth[a] * pow2(64 + delta - hs[a]));
           }
         }
       }
-      wait_job(n);
+      if (n >= early) wait_job(n);
       const uint32_t tl = lanes(n);
       const int nreal = Nb + (PASS != EP_PLANE && A.collision ? g.nf - g.nz : 0);
-      int64_t* exr = ex + a * 8 + rx;
+      int64_t* exr = ex + a * XW + rx;
       for (int q = grp; 4 * q < nreal; q += NG) {
         uint32_t bb[8][4];
         tm_ld(tl + (uint32_t)(4 * q), g.n2, bb);
@@ -723,22 +820,22 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
           // for the weight alone, times 4 for every further factor
           const int64_t w1 = val ? __mul64hi(R[e], wqt[a]) : 0;
           if (f == 0) {
-            moment(jsum + rx, w1);
-            if (KF >= KF_LINEAR) moment(jsum + 8 + rx, __mul64hi(w1, wc));
-            if (KF >= KF_QUADRATIC) moment(jsum + 32 + rx, __mul64hi(__mul64hi(w1, wc), wc));
+            moment<XW>(jsum + rx, w1);
+            if (KF >= KF_LINEAR) moment<XW>(jsum + 8 + rx, __mul64hi(w1, wc));
+            if (KF >= KF_QUADRATIC) moment<XW>(jsum + 32 + rx, __mul64hi(__mul64hi(w1, wc), wc));
           } else if (f < 3) {
             const int64_t w2 = __mul64hi(w1, ws);
-            moment(jsum + 8 * (1 + f) + rx, w2);
-            if (KF >= KF_QUADRATIC) moment(jsum + 8 * (6 + f) + rx, __mul64hi(w2, wc));
+            moment<XW>(jsum + 8 * (1 + f) + rx, w2);
+            if (KF >= KF_QUADRATIC) moment<XW>(jsum + 8 * (6 + f) + rx, __mul64hi(w2, wc));
           } else {
-            moment(jsum + 8 * (2 + f) + rx, __mul64hi(__mul64hi(w1, ws), ws));
+            moment<XW>(jsum + 8 * (2 + f) + rx, __mul64hi(__mul64hi(w1, ws), ws));
           }
         }
       }
       } else {
       // ---- DFS results: rows (b, x); every point is finished here
-      const int b = 16 * (n - g.mt2) + rg;
-      const int w = PASS == EP_PLANE && b >= hb ? rx ^ 4 : rx;
+      const int b = RT * (n - g.mt2) + rg;
+      const int w = PASS == EP_PLANE && b >= hb ? rx ^ XH : rx;
       bool val = b < Nb;
       long long po = 0;   // adjoint: this column's offset in the fields
       double* Kp;
@@ -752,8 +849,8 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
         st = Nb;
         po = o;
       } else {
-        val = val && cur.m0 + (w & 3) < hP;
-        Kp = A.K + cur.base + (long long)b * d.S_l + cur.m0 + (w & 3) + (w >= 4 ? hP : 0);
+        val = val && cur.m0 + (w & (XH - 1)) < hP;
+        Kp = A.K + cur.base + (long long)b * d.S_l + cur.m0 + (w & (XH - 1)) + (w >= XH ? hP : 0);
         Ip = Kp;
         st = (unsigned)d.S_j;
       }
@@ -777,7 +874,7 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
         c0 = A.sgn * t.sinT[cur.k] * t.inv_r[cur.i];
         if (cth_b != b * 64 + cur.m0) {   // cosPh as a fixed-point coefficient of the DFS term
           cth_b = b * 64 + cur.m0;
-          cth = val ? __double2ll_rn(t.cosP[cur.m0 + (w & 3) + (w >= 4 ? hP : 0)] * pow2(62)) : 0;
+          cth = val ? __double2ll_rn(t.cosP[cur.m0 + (w & (XH - 1)) + (w >= XH ? hP : 0)] * pow2(62)) : 0;
         }
       } else {
         c0 = -A.sgn * xc[w];
@@ -824,7 +921,7 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
             const int ha = PASS != EP_PLANE ? hx : hs[a];
             if (PASS != EP_PLANE) W[e] >>= hx;
             else W[e] = __mul64hi(W[e], cth) >> (ha - 2);
-            W[e] += exr[a * 8];
+            W[e] += exr[a * XW];
             qb[e] = qv + ha;
           }
           double y4[4];
@@ -872,13 +969,14 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
       }
       }
       if (PASS == EP_ADJOINT && n >= g.mt2) {
+        if (XW == 4) gks += __shfl_xor_sync(0xFFFFFFFFu, gks, 4);
         gks += __shfl_xor_sync(0xFFFFFFFFu, gks, 8);
         gks += __shfl_xor_sync(0xFFFFFFFFu, gks, 16);
-        if (lane < 8) gp[((n - g.mt2) * (T / 32) + warp) * 8 + lane] = gks;
+        if (lane < XW) gp[((n - g.mt2) * (T / 32) + warp) * 8 + lane] = gks;
       }
       alive = end_job(n);
       if (!alive) break;
-      if (PASS == EP_ADJOINT && n == jobs - 1 && tid < 8 && cur.b0 + tid < d.nblk) {
+      if (PASS == EP_ADJOINT && n == jobs - 1 && tid < XW && cur.b0 + tid < d.nblk) {
         double gt = 0.0;   // the warps' shares in a fixed order
         for (int z = 0; z < g.mt1 * (T / 32); ++z) gt += gp[z * 8 + tid];
         A.gk[cur.b0 + tid] -= gt;
@@ -889,7 +987,8 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
       // moment z of block x as a double (visible after the next wait's barrier)
       const int z = tid >> 3, x = tid & 7;
       constexpr int nm = KF == KF_ISO ? 1 : KF == KF_LINEAR ? 4 : 9;
-      if (z < nm) {
+      if (x >= XW) {
+      } else if (z < nm) {
         // 2 and 4 per factor, as exponents (adjoint: and its weight's)
         const int more = (z == 0 ? 1 : z < 4 ? 3 : 5) + (PASS == EP_ADJOINT ? lgNa : 0);
         const int qv = block_exp(smax[buf * 8 + x]) + m2.se + more;
@@ -955,23 +1054,28 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
   uint32_t* tslot = reinterpret_cast<uint32_t*>(ms + 16);
   volatile int* dead = reinterpret_cast<volatile int*>(ms + 20);   // a wait ran out
   uint32_t* smax = reinterpret_cast<uint32_t*>(ms + 24);   // [2]
-  int* se = reinterpret_cast<int*>(ms + 32);               // [ng * n]
-  double* tot = reinterpret_cast<double*>(ms + 32 + (g.ng * g.n * 4 + 15) / 16 * 16);   // [128]
+  uint64_t* barB = reinterpret_cast<uint64_t*>(ms + 32);   // [2]: a streamed matrix has arrived
+  volatile unsigned* cnt = reinterpret_cast<volatile unsigned*>(ms + 48);  // [3], issuing warp's
+  int* se = reinterpret_cast<int*>(ms + 64);               // [ng * n]
+  double* tot = reinterpret_cast<double*>(ms + 64 + (g.ng * g.n * 4 + 15) / 16 * 16);   // [128]
   double* ts = reinterpret_cast<double*>(sm + g.oA);       // adjoint: [warps][128], before the digits
   if (!g.left || Nr != 8 * g.kc + 1) {   // K paddings read as zero
     for (int x = tid; x < g.oB / 16; x += T)
       reinterpret_cast<uint4*>(sm)[x] = make_uint4(0, 0, 0, 0);
   }
   if (tid < 2) smax[tid] = 0;
+  if (tid < 3) cnt[tid] = 0;
   if (tid == 0) *dead = 0;
   for (int q = 0; q < g.ng; ++q) {
-    copy_in(sm + g.oB + q * g.bB, M.dev[q], g.bB);
+    if (q < g.nb && g.nb == g.ng) copy_in(sm + g.oB + q * g.bB, M.dev[q], g.bB);
     for (int x = tid; x < g.n; x += T) se[q * g.n + x] = M.se[q][x];
   }
   fill_bias(sm + g.oCA, 128);
   if (tid == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(sm_u32(&bar[0])) : "memory");
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(sm_u32(&bar[1])) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(sm_u32(&barB[0])) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(sm_u32(&barB[1])) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -1002,6 +1106,34 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
     base = (long long)(q0 / (unsigned)d.Nt) * d.S_g + (long long)j * d.S_j +
            (long long)l * d.S_l + c0;
   };
+  // Where the matrices do not fit beside the digits they stream through two buffers, in
+  // the order of the groups (T = 512): matrix number z of this CTA goes to buffer z & 1 when the
+  // products of number z - 2 are done. cnt: matrices requested and waited for, the next
+  // one's group (in shared memory: the epilogue needs every register)
+  const bool stream = T == 512 && g.nb != g.ng;
+  auto load_next = [&]() {
+    const unsigned z = cnt[0], q = cnt[2];
+    // the groups of all tiles of this CTA (below 2^31, host)
+    if (z < (unsigned)((A.ntiles - 1 - (long long)blockIdx.x) / gridDim.x + 1) * g.ng) {
+      __syncwarp();
+      if (elect_one()) {
+        const uint32_t br = sm_u32(&barB[z & 1]);
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
+                     :: "r"(br), "r"(g.bB) : "memory");
+        asm volatile(
+            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+            :: "r"(smb + g.oB + (z & 1) * g.bB), "l"(M.dev[q]), "r"(g.bB), "r"(br)
+            : "memory");
+        cnt[0] = z + 1;
+        cnt[2] = q + 1 == (unsigned)g.ng ? 0 : q + 1;
+      }
+      __syncwarp();
+    }
+  };
+  if (stream && uwarp == T / 32 - 1) {
+    load_next();
+    load_next();
+  }
   for (long long tile = blockIdx.x; tile < A.ntiles && alive; tile += gridDim.x, buf ^= 1) {
     int c0;
     long long base;
@@ -1161,7 +1293,16 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
     auto issue = [&](int n) {
       const uint32_t r = g.dual ? (uint32_t)(n & 1) : 0u;
       const uint32_t one = elect_one(), tm = tmem + r * (uint32_t)g.half;
-      const uint32_t ca = smb + g.oCA, a = smb + g.oA, b = smb + g.oB + (uint32_t)(n * g.bB);
+      const uint32_t ca = smb + g.oCA, a = smb + g.oA;
+      uint32_t bq = (uint32_t)n;
+      if (stream) {
+        const unsigned z = __shfl_sync(0xFFFFFFFFu, cnt[1], 0);
+        if (!bar_wait(sm_u32(&barB[z & 1]), (z >> 1) & 1u, p.wait_operand)) *dead = 1;
+        __syncwarp();
+        if (one) cnt[1] = z + 1;
+        bq = z & 1;
+      }
+      const uint32_t b = smb + g.oB + bq * (uint32_t)g.bB;
       if (g.kc == 4)
         chain_steps<2, false, false>(one, tm, ca, a, g.d, g.sb, 0, b, g.left, g.rows, g.n);
       else if (g.kc == 2)
@@ -1228,6 +1369,7 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
       if (!bar_wait(sm_u32(&bar[r]), (phase >> r) & 1u, p.wait_operand)) *dead = 1;
       phase ^= 1u << r;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      if (stream && uwarp == T / 32 - 1 && !*dead) load_next();   // this group's matrix is free
       const uint32_t tl = tmem + r * (uint32_t)g.half + ((uint32_t)((warp & 3) * 32) << 16);
       if (MODE != RAD_ADJOINT && n == 0 && A.tau) {   // the finished rate at the inflow node (both rows lead this group)
         uint32_t b[8][4];
@@ -1304,6 +1446,10 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
           const uint32_t rr = g.dual ? (uint32_t)(x & 1) : 0u;
           bar_wait(sm_u32(&bar[rr]), ((phase >> rr) & 1u) ^ (x == n ? 1u : 0u), kDefaultWaitIters);
         }
+        // and the matrices in flight (the issuing warp's count; full bound)
+        if (stream && uwarp == T / 32 - 1)
+          for (unsigned z = cnt[0] < 2 ? 0 : cnt[0] - 2; z < cnt[0]; ++z)
+            bar_wait(sm_u32(&barB[z & 1]), (uint32_t)(z >> 1) & 1u, kDefaultWaitIters);
         alive = false;
         break;
       }

@@ -19,8 +19,9 @@ struct EmuMat {
   int extra = 0;             // 1: the bias MMA's second core holds a leftover K element's digits
 };
 
-// Geometry of a pass that contracts two axes of a tile of Na x Nb x 8 points.
+// Geometry of a pass that contracts two axes of a tile of Na x Nb x xw points.
 struct EmuGeo {
+  int xw, seq;               // 8 or 4; 1: the two digit copies share their memory
   int Na, Nb, hb;            // DFS axis, Fourier axis, half of the latter
   int ka, kb;                // K cores of 8 along a and b
   int nf, nz;                // functionals of the Fourier operand; nz of them in zero rows
@@ -39,6 +40,7 @@ struct EmuRadGeo {
   int ng, go;                // output groups and outputs per group
   int n, rows;
   int cols, dual, half;
+  int nb;                    // matrix buffers: ng, or 2 that the groups' matrices stream through
   int oA, oB, bB, oCA, oMs, bytes;   // bB: bytes of one group's matrix
   int threads;
 };

@@ -24,6 +24,11 @@ pytestmark = pytest.mark.gpu
 SHAPES = [(3, 2, 2, 2, 2), (5, 3, 2, 6, 4), (9, 5, 4, 8, 6), (16, 4, 6, 10, 8), (17, 8, 8, 8, 8),
           (18, 7, 10, 14, 12), (25, 9, 16, 16, 10), (33, 6, 4, 24, 16), (32, 17, 2, 4, 20),
           (10, 16, 16, 16, 16), (7, 24, 16, 2, 24), (6, 16, 24, 24, 4), (12, 2, 32, 12, 32)]
+# four-wide tiles, with two digit copies and with one (ragged blocks and columns, odd
+# lengths of the DFS axis, one and two DFS tiles); streamed radial matrices
+SHAPES += [(3, 24, 24, 6, 10), (3, 31, 32, 4, 6), (3, 32, 32, 4, 8), (5, 3, 2, 32, 32),
+           (5, 3, 2, 30, 32), (4, 3, 4, 24, 24), (3, 25, 28, 26, 24), (65, 3, 4, 6, 10),
+           (81, 2, 4, 12, 16), (72, 3, 2, 8, 12)]
 
 
 def _rhs(gg, F):

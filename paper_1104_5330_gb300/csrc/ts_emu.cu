@@ -515,9 +515,8 @@ cudaError_t launch2(const Problem& p, const Tables<double>& t, const EmuGeo& g, 
   int ctas = 1;
   const cudaError_t e2 = emu_ctas(T, A.ntiles, &ctas);
   if (e2 != cudaSuccess) return e2;
-  emu::k_emu2<PASS, KF, T, U, NA, NB, XW><<<ctas, T, g.bytes, s>>>(p, t, g, {D.dev, 3 - D.s}, {F.dev, 3 - F.s},
-                                                       A);
-  return cudaGetLastError();
+  return launch_pass(emu::k_emu2<PASS, KF, T, U, NA, NB, XW>, ctas, T, g.bytes, s, p, t, g,
+                     emu::MatArg{D.dev, 3 - D.s}, emu::MatArg{F.dev, 3 - F.s}, A);
 }
 // Units of (a, b) a thread holds: one where the threads cover the tile, else two.
 template <int PASS, int KF>
@@ -630,8 +629,7 @@ cudaError_t launch_rad(const EmuRadGeo& g, const EmuMat* mats, const Problem& p,
     M.dev[q] = mats[q].dev;
     M.se[q] = mats[q].se;
   }
-  emu::k_emu_radial<T, MODE><<<ctas, T, g.bytes, s>>>(p, t, g, M, A);
-  return cudaGetLastError();
+  return launch_pass(emu::k_emu_radial<T, MODE>, ctas, T, g.bytes, s, p, t, g, M, A);
 }
 template <int T>
 cudaError_t launch_rad_mode(const EmuPlan& e, const Problem& p, const Tables<double>& t,

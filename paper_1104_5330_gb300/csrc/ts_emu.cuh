@@ -501,6 +501,7 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                  :: "r"(sm_u32(tslot)), "r"(g.cols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    pass_started();
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -559,6 +560,7 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
     if (KF >= KF_QUADRATIC) cp8(x + 384, p.scc + blk);
     cp8(x + 448, t.sin_th + jj);
   };
+  pass_wait();
   if ((long long)blockIdx.x < A.ntiles) {
     at = tile_at<PASS, XW>(d, blockIdx.x);
     load_units<PASS, U, XW>(d, A.U, at, S, hP, Nb, A.vec, ua, ub, v);
@@ -1082,6 +1084,7 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                  :: "r"(sm_u32(tslot)), "r"(g.cols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    pass_started();
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -1134,6 +1137,7 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
     load_next();
     load_next();
   }
+  pass_wait();
   for (long long tile = blockIdx.x; tile < A.ntiles && alive; tile += gridDim.x, buf ^= 1) {
     int c0;
     long long base;

@@ -22,6 +22,19 @@ namespace ts {
 
 constexpr int kThreads = 256;
 
+// Passes of a step are launched so that the next one may start when every CTA of this
+// one has called pass_started(): its CTAs then take the places that fall free, set up
+// what no field touches (tables, barriers, tensor memory) and wait in pass_wait() until
+// this pass is complete and its writes are visible. Every pass calls pass_wait() before
+// its first access to a field, and, if it allocates tensor memory, pass_started() after
+// that (an allocation never waits for a later pass). Saves 2 to 4 us of a launch.
+__device__ __forceinline__ void pass_started() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void pass_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 template <typename C>
 __device__ __forceinline__ C fmac(C a, C b, C c) { return fma(a, b, c); }
 
@@ -997,6 +1010,8 @@ __device__ __forceinline__ void implicit_collision_tile(const Problem& p, const 
 template <typename T, typename C>
 __global__ void __launch_bounds__(kThreads)
 k_implicit_collision(Problem p, Tables<C> t, T* F, double dt) {
+  pass_started();
+  pass_wait();
   implicit_collision_tile<T, C>(p, t, F, dt, blockIdx.x);
 }
 

@@ -663,7 +663,9 @@ k_angular_pp(Problem p, Tables<C> t, const T* __restrict__ U, T* __restrict__ K,
   C* sSD = su + nb * S;
   C* uT = sSD + nb * ang_ss(NT, NP);
   C* sc = uT + nb * ang_us<C>(NT, NP);
+  pass_started();
   angular_rb_mats<C>(t, d, sP, sQ, sD);
+  pass_wait();
   long long tile = blockIdx.x;
   if (tile < ntiles) angular_rb_load<true, T, C>(d, U, nb, tile, su);
   cp_async_commit();
@@ -859,7 +861,9 @@ k_plane_pp(Problem p, Tables<C> t, const T* __restrict__ U, T* __restrict__ K, C
   C* sD = sQ + Nt * Nt;
   C* buf0 = sD + Np * Np;
   C* sSm = buf0 + 2 * TS;
+  pass_started();
   plane_rb_mats<C>(t, d, sP, sQ, sD);
+  pass_wait();
   long long tile = blockIdx.x;
   if (tile < ntiles) plane_rb_load<true, T, C>(d, U, c, tile, buf0);
   cp_async_commit();
@@ -1146,7 +1150,9 @@ k_plane_sq(Problem p, Tables<C> t, const T* __restrict__ U, T* __restrict__ K, C
   C* sD = sQ + N * N;
   C* buf0 = sD + N * N;
   C* sF = buf0 + 2 * S::TS;
+  pass_started();
   plane_sq_mats<C>(t, d, sP, sQ, sD);
+  pass_wait();
   long long tile = blockIdx.x;
   if (tile < ntiles) plane_sq_load<N, KT, T, C>(d, U, tile, buf0);
   cp_async_commit();
@@ -1536,7 +1542,9 @@ k_radial_eo(Problem p, Tables<C> t, const double* __restrict__ Dr64, const T* U,
   C* sMc = sO + hh4;
   C* sMr = sMc + h4;
   C* sEv = sMr + h4;
+  pass_started();
   radial_rb_mats<C>(t, Nr, sE, sO, sMc, sMr);
+  pass_wait();
   radial_rb_body<Nr_, T, C>(p, t, Dr64, U, Kin, sEv, sE, sO, sMc, sMr, sgn, tau, mode, F, Acc,
                             Uout, out, dt, W, blockIdx.x);
 }

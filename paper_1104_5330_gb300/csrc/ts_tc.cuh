@@ -286,7 +286,9 @@ k_radial_tc(Problem p, Tables<float> t, const void* __restrict__ Bterms, const f
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                  :: "r"(smem_u32(tslot)), "r"(sh.tmem_cols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    pass_started();
   }
+  pass_wait();
   // the tile's N_r lines into shared memory as raw floats, every 16-byte copy in
   // flight at once (cp.async; columns beyond the tile are zero), and the lines
   // of K, F and Acc that the epilogue reads requested into L2 meanwhile

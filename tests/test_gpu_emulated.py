@@ -182,3 +182,26 @@ def test_adjoint_step_matches_the_oracle(n, form):
     lo, gko, geo = op.adjoint_step(F0, lam0, dt)
     for a, b in ((lam, lo), (gk, gko), (ge, geo)):
         assert rel_l2(host(a), b) < 1e-12
+
+
+@pytest.mark.parametrize("precision", ["f64", "f32"])
+def test_captured_step_equals_the_plain_one(precision):
+    """Passes start early outside a capture and are serialised within one."""
+    og, gg, dtype = None, None, torch.float64
+    if precision == "f64":
+        og, gg = pair(0.2, 1.0, 17, 8, 8, 8, 8, G=2)
+    else:
+        dtype = torch.float32
+        og = OGrid(0.2, 1.0, 17, 8, 8, 8, 8, groups=2)
+        gg = T().Grid(0.2, 1.0, 17, 8, 8, 8, 8, groups=2, precision=T().TS_FP32)
+    kap, eta, ks, F0, g1, g2 = absorber_workload(og)
+    gg.set_coeffs(kap, eta, ks, g1, g2)
+    plain, captured = cuda(F0).to(dtype), cuda(F0).to(dtype)
+    gg.step(plain, 1e-4, 3)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        gg.step(captured, 1e-4, 3)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(plain, captured)

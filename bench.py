@@ -14,8 +14,9 @@ runs its own copy of the workload on its own GPU (weak scaling; no collective
 on the data path).
 
 Extra keys: roofline of the dominant kernel (per-launch device time from
-ts_step_profile; FP64 ALU peak derived from the SM count, the FP64 lanes per SM
-and the clock, with a measured DFMA-loop rate beside it), end-to-end rate
+ts_step_profile; in double the f16 digit products against the measured tensor rate,
+with the FP64 pipe's peak, derived from the SM count, the FP64 lanes per SM and the
+clock, and a measured DFMA-loop rate beside it), end-to-end rate
 through ts_step_host (host buffers, copies inside the timed region), the
 reduced-precision variants (FP32, FP32 + FP64 radial rows, tensor-core TF32x3
 and BF16x3) and the adjoint step on the same workload, the same grid with
@@ -880,7 +881,24 @@ def run_ours(args, dims, wname):
     sms = torch.cuda.get_device_properties(local).multi_processor_count
     smax = peaks.get("sm_max_mhz", 2070.0)
     fp64_peak = sms * 2 * FP64_FMA_PER_SM_CLK * smax * 1e6 / 1e12
-    if prec == ts.TS_FP64:
+    if prec == ts.TS_FP64 and os.environ.get("TS_GENERIC_PASSES") != "1":
+        # exact integer products on the tensor cores: eight digits a side, the 36 digit
+        # products of order 0..7 of every dense multiply-add
+        macs = {"angular": 2 * NT + NP, "plane": 2 * Nt + Np, "radial": Nr}[dname]
+        digit_flops = 36 * 2 * macs * pts
+        achieved = digit_flops / (avg_ms * 1e-3) / 1e12
+        roof = {"bound": "tensor", "kernel": "k_emu_radial" if dname == "radial" else "k_emu2",
+                "achieved": achieved, "peak": peaks["bf16_tflops"], "unit": "TFLOP/s",
+                "frac": achieved / peaks["bf16_tflops"], "peak_source": f"{peak_src} bf16_tflops",
+                "limited_by": "integer instructions that cut, recombine and round the digits",
+                "algorithmic_f16_flops_per_launch": digit_flops,
+                "fp64_equivalent_tflops": flops[dname] / (avg_ms * 1e-3) / 1e12,
+                "fp64_pipe_peak_tflops": fp64_peak,
+                "measured_dfma_loop_tflops": ts.ts_probe_fma_rate(ts.TS_FP64),
+                "traffic": _traffic(dname, wname, args.precision),
+                "algorithmic_bytes_per_launch": byts[dname],
+                "hbm_achieved_gbs": byts[dname] / (avg_ms * 1e-3) / 1e9}
+    elif prec == ts.TS_FP64:
         achieved = flops[dname] / (avg_ms * 1e-3) / 1e12
         roof = {"bound": "alu", "kernel": f"{kfam}<double>", "achieved": achieved,
                 "peak": fp64_peak, "unit": "TFLOP/s", "frac": achieved / fp64_peak,

@@ -556,7 +556,9 @@ ts_status ts_stable_dt(ts_grid* grid, const void* x0, int iters, double* rho_hos
  * timeout path: it issues no products, latches the grid's error flag
  * (ts_sync_status then returns TS_ERR_TIMEOUT), waits with the full bound for
  * its own copy to land, frees its tensor memory and returns; that pass's
- * outputs are not written. Only this wait changes: the waits that drain work
+ * outputs are not written. The double-precision passes on the tensor cores bound
+ * their waits for their products the same way: the pass ends early and its outputs
+ * are void. Only these waits change: the waits that drain work
  * in flight keep their full bound. Host-side; takes effect at the next
  * launch. (No counterpart in the paper: a test hook of the bounded waits.) */
 ts_status ts_set_wait_limit(ts_grid* grid, long long operand_wait_iterations);

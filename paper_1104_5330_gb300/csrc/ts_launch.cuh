@@ -239,8 +239,9 @@ cudaError_t Launch<T, C>::angular(const Problem& p, const Tables<C>& t, const T*
       return launch_angular_tc(p, t, U, K, sgn, collision, s);
   }
   // double precision: exact integer products on the tensor cores wherever the tile fits
-  // (33 x 16^4 x 4: angular 440 -> 125 us, plane 386 -> 119, radial 381 -> 144; also the
-  // faster one on the smallest grids, 17 x 8^4: 25, 19, 21 -> 13, 12, 15)
+  // (33 x 16^4 x 4: angular 440 -> 128 us, plane 386 -> 121, radial 381 -> 144; 65 x 32^4: a
+  // step 77.9 -> 17.8 ms; also the faster one on the smallest grids, 17 x 8^4: 25, 19, 21
+  // -> 13, 13, 15)
   if constexpr (sizeof(T) == 8) {
     if (p.emu && emu_has_angular(*p.emu, d))
       return emu_angular(*p.emu, p, t, false, U, K, sgn, collision, s);

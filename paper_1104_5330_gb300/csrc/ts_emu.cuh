@@ -1290,6 +1290,15 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
         }
       }
     }
+    // every thread of a column reads the inflow node's rate before the barrier: the
+    // right-hand side writes over its own Kin, and one of them stores that node first
+    const bool val = row < Wc;
+    const int kT = val ? (c0 + row) / NP : 0;
+    const double cT = t.cosT[kT], ck = A.sgn * cT;
+    const int bn = cT > 0.0 ? 0 : N;   // inflow node
+    const double* Kc = A.Kin + base + row;
+    const unsigned Si = (unsigned)d.S_i;   // a group spans less than 2^32 elements (host)
+    double kb = MODE != RAD_ADJOINT && val && A.tau ? Kc[(unsigned)bn * Si] : 0.0;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -1321,15 +1330,8 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
       __syncwarp();
     };
     int issued = 0;
-    const bool val = row < Wc;
-    const int kT = val ? (c0 + row) / NP : 0;
-    const double cT = t.cosT[kT], ck = A.sgn * cT;
-    const int bn = cT > 0.0 ? 0 : N;   // inflow node
-    const double* Kc = A.Kin + base + row;
     const double* Fc = A.F + base + row;
     const double* Ac = A.Acc + base + row;
-    const unsigned Si = (unsigned)d.S_i;   // a group spans less than 2^32 elements (host)
-    double kb = MODE != RAD_ADJOINT && val && A.tau ? Kc[(unsigned)bn * Si] : 0.0;
     double* dst = (MODE == RAD_RHS || MODE == RAD_ADJOINT ? A.out
                    : MODE == RAD_STAGE3 || MODE == RAD_AB2 || MODE == RAD_AB2_START ? A.F
                                                                                     : A.Uout) +

@@ -1,0 +1,46 @@
+"""ts_rhs writes the finished rate over the array that holds the angular and plane terms.
+Every thread of a radial line needs the inflow node's entry of that array (the Tau rows),
+so it has to be read before any thread of the line stores that node.
+
+The derivative that an AB2 start step forms from the same input does not write over what
+it reads. With dt = 2^200 (float: 2^60) the step's field is that derivative times dt, bit
+for bit, wherever it is not zero: the field itself is below half a unit of the last place.
+"""
+import pytest
+import torch
+
+from gpu_common import T, absorber_workload, cuda, host, pair, rel_l2
+from oracle.transport import Problem as OProblem
+
+pytestmark = pytest.mark.gpu
+
+
+def _equal_to_the_start_step(precision, power, n, calls):
+    ts = T()
+    dims = (0.2, 1.0) + n
+    dtype = torch.float64 if precision == ts.TS_FP64 else torch.float32
+    og, rhs = pair(*dims, G=2, precision=precision)
+    ab2 = ts.Grid(*dims, groups=2, precision=precision, scheme=ts.TS_AB2)
+    kap, eta, ks, F0, g1, g2 = absorber_workload(og)
+    for g in (rhs, ab2):
+        g.set_coeffs(kap, eta, ks, g1, g2)
+    F = cuda(F0).to(dtype)
+    step = F.clone()
+    ab2.step(step, 2.0 ** power, 1)
+    K = torch.empty_like(F)
+    for _ in range(calls):
+        K.fill_(float("nan"))
+        ts.ts_rhs(rhs.handle, F, K)
+        ts.ts_sync_status(rhs.handle)
+        some = K != 0
+        assert float(some.double().mean()) > 0.9
+        assert torch.equal(K[some] * 2.0 ** power, step[some])
+    return host(K), OProblem(og, kap, eta, ks, g1, g2).rhs(F0)
+
+
+# two and four threads a line, one to three output groups, streamed matrices, partial tiles
+@pytest.mark.parametrize("n", [(17, 4, 6, 8, 12), (33, 3, 4, 16, 16), (65, 2, 4, 10, 12),
+                               (81, 2, 2, 8, 16)], ids=str)
+def test_double_precision(n):
+    K, ref = _equal_to_the_start_step(T().TS_FP64, 200, n, 20)
+    assert rel_l2(K, ref) < 1e-12

@@ -366,6 +366,16 @@ k_radial_tc(Problem p, Tables<float> t, const void* __restrict__ Bterms, const f
     }
     __syncwarp();
   }
+  // this thread's column (TMEM lane w; two threads a column). Both read the inflow node's
+  // rate before the barriers: the right-hand side writes over its own Kin, and one of them
+  // stores that node
+  const int w = tid & 127, half = tid >> 7;
+  const bool act = w < Wc;
+  const int k = act ? (c0 + w) / NP : 0;
+  const int b = t.cosT[k] > 0.f ? 0 : Nr - 1;
+  const long long Si = d.S_i;
+  const float* Kc = Kin + base + w;   // this column's lines
+  const float k0 = act ? Kc[(long long)b * Si] : 0.f;
   // every thread waits for the products (bounded); `issued` is CTA-wide: the
   // MMAs and their commit were issued only if thread 0's operand wait succeeded
   const bool issued = __syncthreads_and(ok ? 1 : 0);
@@ -383,22 +393,16 @@ k_radial_tc(Problem p, Tables<float> t, const void* __restrict__ Bterms, const f
     // reading the products from TMEM 8 rows at a time (the loads of a warp are
     // issued by all its lanes); the loads of each group are all issued before
     // any of its stores
-    const int w = tid & 127, half = tid >> 7;
     const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    const bool act = w < Wc;
-    const int k = act ? (c0 + w) / NP : 0;
     const float ck = sgn * t.cosT[k];
-    const int b = t.cosT[k] > 0.f ? 0 : Nr - 1;
     float dv[8];
     tmem_ld8(lane_base + (uint32_t)((Nr - 1) / 8 * 8), dv);   // group holding row N
     const float dN = dv[(Nr - 1) % 8];
     tmem_ld8(lane_base, dv);                                  // group holding row 0
     const float db = b == 0 ? dv[0] : dN;
-    const long long Si = d.S_i;
-    const float* Kc = Kin + base + w;   // this column's lines
     const float* Fc = F + base + w;
     const float* Ac = Acc + base + w;
-    const float kb = act ? Kc[(long long)b * Si] + ck * db : 0.f;
+    const float kb = act ? k0 + ck * db : 0.f;
     const float tb = t.tsign[b];
     // every update mode as dst = f + cv (cw v + ca ac), Acc = aa ac + ab v
     const bool rhs = mode == RAD_RHS;

@@ -44,3 +44,11 @@ def _equal_to_the_start_step(precision, power, n, calls):
 def test_double_precision(n):
     K, ref = _equal_to_the_start_step(T().TS_FP64, 200, n, 20)
     assert rel_l2(K, ref) < 1e-12
+
+
+# split TF32 and split bf16: two threads a line
+@pytest.mark.parametrize("n", [(17, 4, 6, 8, 16), (33, 3, 4, 16, 16), (41, 2, 4, 8, 24)], ids=str)
+@pytest.mark.parametrize("precision", ["TS_TF32X3", "TS_BF16X3"])
+def test_split_products(precision, n):
+    K, ref = _equal_to_the_start_step(getattr(T(), precision), 60, n, 20)
+    assert rel_l2(K, ref) < 1e-5

@@ -473,7 +473,6 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
   unsigned char* ms = sm + g.oMs;
   uint64_t* bar = reinterpret_cast<uint64_t*>(ms);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(ms + 16);
-  volatile int* dead = reinterpret_cast<volatile int*>(ms + 20);  // a wait ran out
   uint32_t* smax = reinterpret_cast<uint32_t*>(ms + 32);          // [2][8]
   double* xs = reinterpret_cast<double*>(ms + 96);                // [2][8][8] scalars of a tile's x
   double* xm = xs + 2 * 64;                                       // [10][8] moments
@@ -488,7 +487,6 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
       reinterpret_cast<uint4*>(sm)[x] = make_uint4(0, 0, 0, 0);
   }
   if (tid < 16) smax[tid] = 0;
-  if (tid == 0) *dead = 0;
   copy_in(sm + g.oB1, m1.dev, (1 + g.kc1) * g.r1 * 16);
   copy_in(sm + g.oB2, m2.dev, (1 + g.kc2) * g.r2 * 16);
   fill_bias(sm + g.oCA, 128);
@@ -572,7 +570,7 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
   int cth_b = -1;    // plane: cosPh of its DFS rows, and of which
   int64_t cth = 0;
   uint32_t phase = 0;   // one bit per barrier
-  bool alive = true;
+  bool alive = true, late = false;   // late: a wait of this thread ran out
   int buf = 0;
   for (long long tile = blockIdx.x; tile < A.ntiles && alive; tile += gridDim.x, buf ^= 1) {
     // ---- largest magnitude of each block (angular) or of the tile (plane)
@@ -703,18 +701,19 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
     int issued = 0;
     const int early = XW == 4 && g.seq ? g.mt2 : 0;   // jobs waited for ahead of their epilogue
     // waits for job n, every warp for itself; where a wait runs out the warp goes on (its
-    // results are void) and all leave together after the job's barrier
+    // results are void) and all leave together: the job's barrier takes the vote (a flag in
+    // shared memory could be set by the next job's waits before the last thread reads it)
     auto wait_job = [&](int n) {
       const uint32_t r = g.dual ? (uint32_t)(n & 1) : 0u;
-      if (!bar_wait(sm_u32(&bar[r]), (phase >> r) & 1u, p.wait_operand)) *dead = 1;
+      late |= !bar_wait(sm_u32(&bar[r]), (phase >> r) & 1u, p.wait_operand);
       phase ^= 1u << r;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     };
     auto end_job = [&](int n) {
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncthreads();
+      const bool over = __syncthreads_or(late ? 1 : 0);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      if (*dead) {
+      if (over) {
         if (tid == 0 && p.err) atomicExch(p.err, 1);
         // our own MMAs end before the CTA exits (full bound)
         for (int x = n; x < issued; ++x) {
@@ -1054,7 +1053,6 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
   unsigned char* ms = sm + g.oMs;
   uint64_t* bar = reinterpret_cast<uint64_t*>(ms);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(ms + 16);
-  volatile int* dead = reinterpret_cast<volatile int*>(ms + 20);   // a wait ran out
   uint32_t* smax = reinterpret_cast<uint32_t*>(ms + 24);   // [2]
   uint64_t* barB = reinterpret_cast<uint64_t*>(ms + 32);   // [2]: a streamed matrix has arrived
   volatile unsigned* cnt = reinterpret_cast<volatile unsigned*>(ms + 48);  // [3], issuing warp's
@@ -1067,7 +1065,6 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
   }
   if (tid < 2) smax[tid] = 0;
   if (tid < 3) cnt[tid] = 0;
-  if (tid == 0) *dead = 0;
   for (int q = 0; q < g.ng; ++q) {
     if (q < g.nb && g.nb == g.ng) copy_in(sm + g.oB + q * g.bB, M.dev[q], g.bB);
     for (int x = tid; x < g.n; x += T) se[q * g.n + x] = M.se[q][x];
@@ -1096,7 +1093,7 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
   // MODE: the update; RAD_STAGE1 stands for stages 1 and 2 (A.mode tells them apart)
   constexpr bool rA = MODE == RAD_STAGE1 || MODE == RAD_STAGE3 || MODE == RAD_AB2;
   uint32_t phase = 0;
-  bool alive = true;
+  bool alive = true, late = false;   // late: a wait of this thread ran out
   int buf = 0;
   constexpr int U = 3;   // (node, 8 columns) units held per thread and round
   auto coords = [&](long long tile, int& c0, long long& base) {
@@ -1310,7 +1307,7 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
       uint32_t bq = (uint32_t)n;
       if (stream) {
         const unsigned z = __shfl_sync(0xFFFFFFFFu, cnt[1], 0);
-        if (!bar_wait(sm_u32(&barB[z & 1]), (z >> 1) & 1u, p.wait_operand)) *dead = 1;
+        late |= !bar_wait(sm_u32(&barB[z & 1]), (z >> 1) & 1u, p.wait_operand);
         __syncwarp();
         if (one) cnt[1] = z + 1;
         bq = z & 1;
@@ -1371,11 +1368,12 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
       const int no = min(g.go, Nr - n * g.go);
       if (4 * grp < no) load_rows(n, grp, no);
       // where a wait runs out the warp goes on (its results are void) and all leave
-      // together after the group's barrier
-      if (!bar_wait(sm_u32(&bar[r]), (phase >> r) & 1u, p.wait_operand)) *dead = 1;
+      // together: the group's barrier takes the vote
+      late |= !bar_wait(sm_u32(&bar[r]), (phase >> r) & 1u, p.wait_operand);
       phase ^= 1u << r;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      if (stream && uwarp == T / 32 - 1 && !*dead) load_next();   // this group's matrix is free
+      if (stream && uwarp == T / 32 - 1 && !__any_sync(0xFFFFFFFFu, late))
+        load_next();   // this group's matrix is free
       const uint32_t tl = tmem + r * (uint32_t)g.half + ((uint32_t)((warp & 3) * 32) << 16);
       if (MODE != RAD_ADJOINT && n == 0 && A.tau) {   // the finished rate at the inflow node (both rows lead this group)
         uint32_t b[8][4];
@@ -1444,9 +1442,9 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
         }
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncthreads();
+      const bool over = __syncthreads_or(late ? 1 : 0);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      if (*dead) {
+      if (over) {
         if (tid == 0 && p.err) atomicExch(p.err, 1);
         for (int x = n; x < issued; ++x) {   // our own MMAs end first (full bound)
           const uint32_t rr = g.dual ? (uint32_t)(x & 1) : 0u;

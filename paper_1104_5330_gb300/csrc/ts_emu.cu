@@ -294,10 +294,11 @@ bool geometry_radial(int Nr, EmuRadGeo* out) {
       g.oA = take(8 * g.d + 256);
       g.oB = take(g.nb * g.bB);
       g.oCA = take(2 * 128 * 16);
-      g.oMs = take(64 + (ng * g.n * 4 + 15) / 16 * 16 + 128 * 8);
+      g.oMs = take(64 + (ng * g.n * 4 + 15) / 16 * 16 + 128 * 8 + 2 * 128 * 4);
       g.bytes = o;
       if (g.bytes > (two ? kTwoCtas : kOneCta)) continue;
       g.threads = two ? 256 : 512;
+      if (Nr * 16 > kEmuRadUnits * g.threads) continue;
       g.half = pow2_at_least(reg);
       g.dual = g.half <= (two ? 128 : 256) && ng > 1;
       g.cols = g.dual ? 2 * g.half : g.half;
@@ -451,8 +452,7 @@ EmuPlan* emu_create(const ts_grid_desc& g, cudaError_t* err) {
     const EmuRadGeo& r = e->gRad;
     const std::vector<Wide> Dr = cheb_wide(Nr, g.R1, g.R2);
     e->rad = true;
-    // the transposed pass keeps a tile's values in registers
-    e->radT = adj && Nr * 16 <= 3 * r.threads;
+    e->radT = adj;
     for (int tr = 0; tr < 2; ++tr) {
       bool& ok = tr ? e->radT : e->rad;
       for (int q = 0; q < r.ng && ok; ++q) {

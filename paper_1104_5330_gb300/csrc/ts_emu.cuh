@@ -265,6 +265,22 @@ __device__ __forceinline__ uint32_t slow_limit(int qb) {
   return (uint32_t)(qb - 1) > 1900u ? 0xFFFFFFFFu : 1u;
 }
 
+// A line's key is its largest exponent and a mantissa of ones, 0 for a line of zeros (values
+// below 2^-1042 count as such). Nothing is cut relative to less than kLeastKey; lines below
+// that, if they are not zero, are scaled up by 2^256 first (tiny_key), and their key says
+// so in its last bit.
+constexpr uint32_t kLeastKey = 64u << 20 | 0xFFFFFu;
+__device__ __forceinline__ uint32_t line_key(uint32_t mx) { return mx ? mx | 0xFFFFFu : 0u; }
+__device__ __forceinline__ bool tiny_line(uint32_t mx) { return mx - 1u < (64u << 20) - 1u; }
+__device__ __forceinline__ uint32_t tiny_key(uint32_t key) {
+  return (max(key >> 20, 1u) + 257u) << 20 | 0xFFFFEu;
+}
+// The exponent base of a line, 5000 with an infinity or a NaN.
+__device__ __forceinline__ int line_exp(uint32_t key) {
+  const int e = (int)(key >> 20);
+  return key == 0 ? 64 : !(key & 1u) ? e - 256 : e == 2047 ? 5000 : max(e, 64);
+}
+
 // The fixed-point key of a block: its largest exponent, at least 64, and a mantissa of ones.
 __device__ __forceinline__ uint32_t fixed_key(uint32_t mx) {
   return ((uint32_t)max((int)(mx >> 20), 64) << 20) | 0xFFFFFu;
@@ -1018,7 +1034,11 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
 // ============================================================================
 // Radial pass: 128 (Theta, Phi) columns of one (g, theta, phi) per tile, all N_r
 // nodes. Digits [digit][column / 8][node][8 columns], MN-major; the matrix rows
-// are ordered 0, N, 1, 2, ..., N-1 so that the two Tau rows come first.
+// are ordered 0, N, 1, 2, ..., N-1 so that the two Tau rows come first. Every line is cut
+// relative to its own largest magnitude (a column is a row of the product, so the scale
+// joins in the epilogue): lines of one tile do not meet in this pass, and a faint direction
+// beside a beam keeps its digits. One scale for the tile was no faster (33 x 16^4 x 4: 1471
+// us a step with it, 1472 without).
 struct RadArgs {
   const double *U, *Kin;
   double sgn;
@@ -1053,17 +1073,19 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
   unsigned char* ms = sm + g.oMs;
   uint64_t* bar = reinterpret_cast<uint64_t*>(ms);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(ms + 16);
-  uint32_t* smax = reinterpret_cast<uint32_t*>(ms + 24);   // [2]
+  volatile uint32_t* tiny = reinterpret_cast<volatile uint32_t*>(ms + 24);   // [2] a line is
   uint64_t* barB = reinterpret_cast<uint64_t*>(ms + 32);   // [2]: a streamed matrix has arrived
   volatile unsigned* cnt = reinterpret_cast<volatile unsigned*>(ms + 48);  // [3], issuing warp's
   int* se = reinterpret_cast<int*>(ms + 64);               // [ng * n]
   double* tot = reinterpret_cast<double*>(ms + 64 + (g.ng * g.n * 4 + 15) / 16 * 16);   // [128]
+  uint32_t* ckey = reinterpret_cast<uint32_t*>(tot + 128);   // [2][128] keys of the lines
   double* ts = reinterpret_cast<double*>(sm + g.oA);       // adjoint: [warps][128], before the digits
   if (!g.left || Nr != 8 * g.kc + 1) {   // K paddings read as zero
     for (int x = tid; x < g.oB / 16; x += T)
       reinterpret_cast<uint4*>(sm)[x] = make_uint4(0, 0, 0, 0);
   }
-  if (tid < 2) smax[tid] = 0;
+  if (tid < 256) ckey[tid] = 0;
+  if (tid < 2) tiny[tid] = 0;
   if (tid < 3) cnt[tid] = 0;
   for (int q = 0; q < g.ng; ++q) {
     if (q < g.nb && g.nb == g.ng) copy_in(sm + g.oB + q * g.bB, M.dev[q], g.bB);
@@ -1095,7 +1117,7 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
   uint32_t phase = 0;
   bool alive = true, late = false;   // late: a wait of this thread ran out
   int buf = 0;
-  constexpr int U = 3;   // (node, 8 columns) units held per thread and round
+  constexpr int U = kEmuRadUnits;   // (node, 8 columns) units held per thread: all of them
   auto coords = [&](long long tile, int& c0, long long& base) {
     unsigned q0 = (unsigned)tile;   // tiles of a field fit 32 bits (checked on the host)
     c0 = (int)(q0 % (unsigned)nch) * 128;
@@ -1151,10 +1173,10 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
         if (rA) prefetch_line(A.Acc + gi);
       }
     }
-    // the tile's values, and their largest magnitude; U units a thread are kept in
-    // registers (longer lines are read again for the conversion)
+    // the tile's values, and the largest magnitude of every line: all units of a thread hold
+    // the same eight lines
     double v[U][8];
-    uint32_t mx = 0;
+    uint32_t mx[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     auto load_unit = [&](int u, double (&z)[8]) {
       const int w = (u & 15) * 8;
 #pragma unroll
@@ -1179,8 +1201,8 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
     for (int q = 0; q < U; ++q) load_unit(tid + q * T, v[q]);
     if (MODE == RAD_ADJOINT) {
       // lt = Tau^T (scale X): every row but the inflow one as it is, that one less
-      // T_N(x_b) sum_i T_N(x_i) X_i. The units hold all nodes (host): a thread's share
-      // of its eight columns' sums, then the half warps', then the CTA's, in fixed order
+      // T_N(x_b) sum_i T_N(x_i) X_i: a thread's share of its eight columns' sums, then the
+      // half warps', then the CTA's, in fixed order
 #pragma unroll
       for (int q = 0; q < U; ++q)
 #pragma unroll
@@ -1239,52 +1261,68 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
     for (int q = 0; q < U; ++q)
 #pragma unroll
       for (int x = 0; x < 8; ++x)
-        mx = max(mx, (uint32_t)__double2hiint(v[q][x]) & 0x7FFFFFFFu);
-    for (int u = tid + U * T; u < Nr * 16; u += T) {
-      double z[8];
-      load_unit(u, z);
+        mx[x] = max(mx[x], (uint32_t)__double2hiint(v[q][x]) & 0x7FFFFFFFu);
+    bool low = false;
 #pragma unroll
-      for (int x = 0; x < 8; ++x) mx = max(mx, (uint32_t)__double2hiint(z[x]) & 0x7FFFFFFFu);
+    for (int x = 0; x < 4; ++x) {   // the half warps hold the same lines: four each
+      const uint32_t send = lane & 16 ? mx[x] : mx[x + 4], keep = lane & 16 ? mx[x + 4] : mx[x];
+      const uint32_t r = max(keep, __shfl_xor_sync(0xFFFFFFFFu, send, 16));
+      low |= tiny_line(r);
+      atomicMax(&ckey[buf * 128 + (lane & 15) * 8 + x + (lane & 16) / 4], line_key(r));
     }
-    mx = __reduce_max_sync(0xFFFFFFFFu, mx);
-    if (lane == 0) atomicMax(&smax[buf], mx);
+    if (low) tiny[buf] = 1;   // (another node of the line may be larger)
     __syncthreads();
-    if (tid == 0) smax[buf ^ 1] = 0;
-    const uint32_t tmax = smax[buf], EM = fixed_key(tmax);
-    const int eb = block_exp(tmax);
-    for (int u0 = tid; u0 < Nr * 16; u0 += U * T) {
-      if (u0 != tid) {
+    if (tid < 128) ckey[(buf ^ 1) * 128 + tid] = 0;
+    if (tid == 128) tiny[buf ^ 1] = 0;
+    const uint32_t* keys = ckey + buf * 128 + (tid & 15) * 8;   // of this thread's lines
+    const bool up = tiny[buf] != 0;
+    auto lift = [&](double (&z)[8]) {   // brings the values of tiny lines up
 #pragma unroll
-        for (int q = 0; q < U; ++q) load_unit(u0 + q * T, v[q]);
+      for (int x = 0; x < 8; ++x)
+        if (!(keys[x] & 1u)) z[x] *= pow2(256);
+    };
+    if (up) {
+      __syncthreads();
+      if (tid < 128) {
+        const uint32_t key = ckey[buf * 128 + tid];
+        if (key != 0 && key < kLeastKey) ckey[buf * 128 + tid] = tiny_key(key);
       }
+      __syncthreads();
+    }
 #pragma unroll
-      for (int q = 0; q < U; ++q) {
-        const int u = u0 + q * T;
-        if (u >= Nr * 16) continue;
-        const int ii = u >> 4, wg = u & 15;
-        uint64_t f[8];
+    for (int q = 0; q < U; ++q) {
+      const int u = tid + q * T;
+      if (u >= Nr * 16) continue;
+      const int ii = u >> 4, wg = u & 15;
+      if (up) lift(v[q]);
+      uint64_t f[8];
 #pragma unroll
-        for (int x = 0; x < 8; ++x) f[x] = to_fixed(v[q][x], EM);
-        if (g.left && ii == N) {
-          // the leftover node: its eight digits beside the bias, one 16-byte row per column
+      for (int x = 0; x < 8; x += 4) {
+        const uint4 k = *reinterpret_cast<const uint4*>(keys + x);
+        f[x] = to_fixed(v[q][x], max(k.x, kLeastKey));
+        f[x + 1] = to_fixed(v[q][x + 1], max(k.y, kLeastKey));
+        f[x + 2] = to_fixed(v[q][x + 2], max(k.z, kLeastKey));
+        f[x + 3] = to_fixed(v[q][x + 3], max(k.w, kLeastKey));
+      }
+      if (g.left && ii == N) {
+        // the leftover node: its eight digits beside the bias, one 16-byte row per column
 #pragma unroll
-          for (int x = 0; x < 8; ++x) {
-            const uint32_t lo = (uint32_t)f[x], hi = (uint32_t)(f[x] >> 32);
-            *reinterpret_cast<uint4*>(sm + g.oCA + 2048 + (wg * 8 + x) * 16) =
-                make_uint4(__byte_perm(hi, 0, 0x4243), __byte_perm(hi, 0, 0x4041),
-                           __byte_perm(lo, 0, 0x4243), __byte_perm(lo, 0, 0x4041));
-          }
-          continue;
+        for (int x = 0; x < 8; ++x) {
+          const uint32_t lo = (uint32_t)f[x], hi = (uint32_t)(f[x] >> 32);
+          *reinterpret_cast<uint4*>(sm + g.oCA + 2048 + (wg * 8 + x) * 16) =
+              make_uint4(__byte_perm(hi, 0, 0x4243), __byte_perm(hi, 0, 0x4041),
+                         __byte_perm(lo, 0, 0x4243), __byte_perm(lo, 0, 0x4041));
         }
-        unsigned char* c = sm + g.oA + wg * g.sb + ii * 16;
+        continue;
+      }
+      unsigned char* c = sm + g.oA + wg * g.sb + ii * 16;
 #pragma unroll
-        for (int w = 3; w >= 0; --w) {
-          uint32_t pk[4];
-          pack_pairs(f, w, pk);
+      for (int w = 3; w >= 0; --w) {
+        uint32_t pk[4];
+        pack_pairs(f, w, pk);
 #pragma unroll
-          for (int h = 0; h < 2; ++h)
-            *reinterpret_cast<uint4*>(c + (7 - (2 * w + h)) * g.d) = digit_of(pk, h);
-        }
+        for (int h = 0; h < 2; ++h)
+          *reinterpret_cast<uint4*>(c + (7 - (2 * w + h)) * g.d) = digit_of(pk, h);
       }
     }
     // every thread of a column reads the inflow node's rate before the barrier: the
@@ -1327,6 +1365,7 @@ k_emu_radial(Problem p, Tables<double> t, EmuRadGeo g, RadMats M, RadArgs A) {
       __syncwarp();
     };
     int issued = 0;
+    const int eb = line_exp(ckey[buf * 128 + row]);
     const double* Fc = A.F + base + row;
     const double* Ac = A.Acc + base + row;
     double* dst = (MODE == RAD_RHS || MODE == RAD_ADJOINT ? A.out

@@ -34,6 +34,8 @@ struct EmuGeo {
   int threads;
 };
 
+constexpr int kEmuRadUnits = 3;   // (node, 8 columns) units of a tile that a thread holds
+
 struct EmuRadGeo {
   int Nr, kc, left;          // K cores; 1: node N_r - 1 rides in the bias MMA
   int sb, d;                 // row group and digit strides of the digits

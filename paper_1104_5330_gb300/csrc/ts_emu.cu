@@ -187,7 +187,7 @@ constexpr int kTwoCtas = 113 * 1024;   // shared memory of each of two CTAs on a
 constexpr int kOneCta = 227 * 1024;
 
 bool geometry2_form(int xw, bool seq, int Na, int Nb, const EmuMat& D, const EmuMat& F, int nf,
-                    int nz, EmuGeo* out) {
+                    int nz, bool adj, EmuGeo* out) {
   EmuGeo g{};
   g.xw = xw;
   g.seq = seq ? 1 : 0;
@@ -229,7 +229,10 @@ bool geometry2_form(int xw, bool seq, int Na, int Nb, const EmuMat& D, const Emu
   g.oB2 = take(F.bytes());
   g.oCA = take(2 * 128 * 16);
   g.oEx = alias ? g.oC2 : take(exB);
-  g.oMs = take(96 + (128 + 160 + Na + g.mt1 * 16 * 8) * 8);
+  // header, scalars, moments; angular: weights and shares; plane: shifts
+  const int kf = nf >= 5 ? 2 : nf >= 3 ? 1 : 0;
+  const int shares = std::max(4 * emu_moments(kf), adj ? g.mt1 * 16 : 0) * 8;
+  g.oMs = take(96 + (128 + 80 + (nf ? emu_weights(kf) * Na + shares : Na)) * 8);
   // a 128-row tile may read row groups past the last one: inside the allocation
   const int over = std::max(g.oC1 + 7 * g.d1 + (16 * g.mt1 + hg) * g.sb1 + 256,
                             g.oC2 + 7 * g.d2 + 16 * g.mt2 * g.sb2 + 256);
@@ -256,11 +259,12 @@ bool geometry2_form(int xw, bool seq, int Na, int Nb, const EmuMat& D, const Emu
 }
 // Eight x where both copies fit; else four (which need whole pairs in each half of the
 // Fourier axis), with the copies in one buffer if need be.
-bool geometry2(int Na, int Nb, const EmuMat& D, const EmuMat& F, int nf, int nz, EmuGeo* out) {
-  if (geometry2_form(8, false, Na, Nb, D, F, nf, nz, out)) return true;
+bool geometry2(int Na, int Nb, const EmuMat& D, const EmuMat& F, int nf, int nz, bool adj,
+               EmuGeo* out) {
+  if (geometry2_form(8, false, Na, Nb, D, F, nf, nz, adj, out)) return true;
   if (Nb % 4) return false;
-  return geometry2_form(4, false, Na, Nb, D, F, nf, nz, out) ||
-         geometry2_form(4, true, Na, Nb, D, F, nf, nz, out);
+  return geometry2_form(4, false, Na, Nb, D, F, nf, nz, adj, out) ||
+         geometry2_form(4, true, Na, Nb, D, F, nf, nz, adj, out);
 }
 
 bool geometry_radial(int Nr, EmuRadGeo* out) {
@@ -377,18 +381,17 @@ EmuPlan* emu_create(const ts_grid_desc& g, cudaError_t* err) {
       mF[NP + 4][q] = c * s;
     }
     e->ang = add_matrix(mD, dfs_order(NT), -1, true, &e->angD, &up);
-    const int nf[kEmuForms] = {1, 3, 5};
     for (int f = 0; f < kEmuForms && e->ang; ++f) {
       // sinPh vanishes at Phi = 0 and pi: the first functionals take those rows of the
       // advective form, the others follow behind the derivatives
-      const int nz = cons ? 0 : std::min(nf[f], 2);
+      const int nf = emu_functionals(f), nz = cons ? 0 : std::min(nf, 2);
       Mat part(mF.begin(), mF.begin() + NP);
-      for (int q = 0; q < nf[f]; ++q) {
+      for (int q = 0; q < nf; ++q) {
         if (q < nz) part[q * (NP / 2)] = mF[NP + q];
         else part.push_back(mF[NP + q]);
       }
       e->ang = add_matrix(part, plain_order(NP, (NP + 15) / 16 * 2), -1, true, &e->angF[f], &up) &&
-               geometry2(NT, NP, e->angD, e->angF[f], nf[f], nz, &e->gAng[f]);
+               geometry2(NT, NP, e->angD, e->angF[f], nf, nz, false, &e->gAng[f]);
     }
   }
   const bool adj = !cons && g.radial == TS_RADIAL_CHEBYSHEV;   // the forms that have an adjoint
@@ -413,11 +416,11 @@ EmuPlan* emu_create(const ts_grid_desc& g, cudaError_t* err) {
       mF[NP + 4][m] = c * s;
     }
     e->adj = add_matrix(mD, dfs_order(NT), -1, true, &e->adjD, &up);
-    const int nf[kEmuForms] = {1, 3, 5};
     for (int f = 0; f < kEmuForms && e->adj; ++f) {
-      Mat part(mF.begin(), mF.begin() + NP + nf[f]);
+      const int nf = emu_functionals(f);
+      Mat part(mF.begin(), mF.begin() + NP + nf);
       e->adj = add_matrix(part, plain_order(NP, (NP + 15) / 16 * 2), -1, true, &e->adjF[f], &up) &&
-               geometry2(NT, NP, e->adjD, e->adjF[f], nf[f], 0, &e->gAdj[f]);
+               geometry2(NT, NP, e->adjD, e->adjF[f], nf, 0, true, &e->gAdj[f]);
     }
   }
   {
@@ -432,7 +435,7 @@ EmuPlan* emu_create(const ts_grid_desc& g, cudaError_t* err) {
       for (int q = 0; q < Np; ++q) mF[l][q] = Dp[(size_t)l * Np + q];
     e->plane = add_matrix(mD, dfs_order(Nt), -1, true, &e->plD, &up) &&
                add_matrix(mF, plain_order(Np, (Np + 15) / 16 * 2), -1, true, &e->plF, &up) &&
-               geometry2(Nt, Np, e->plD, e->plF, 0, 0, &e->gPl);
+               geometry2(Nt, Np, e->plD, e->plF, 0, 0, false, &e->gPl);
     if (adj && e->plane) {
       // transposed: a_th changes sign at the partner (cos(Ph + pi) = -cosPh), so it comes
       // out of the contraction with the partner's matrix negated

@@ -259,6 +259,12 @@ __device__ __forceinline__ void to_double4(const int64_t (&R)[4], const int (&qb
       if (top[e] < lim) y[e] = to_double_slow(R[e], qb[e]);
   }
 }
+__device__ __forceinline__ uint32_t slow_limit(int qb);
+__device__ __forceinline__ double to_double1(int64_t R, int qb) {
+  uint32_t top;
+  const double y = to_double_fast(R, (qb + 62) << 20, top);
+  return top < slow_limit(qb) ? to_double_slow(R, qb) : y;
+}
 // 2^n as a double, -1022 < n < 1023
 __device__ __forceinline__ double pow2(int n) { return __hiloint2double((1023 + n) << 20, 0); }
 __device__ __forceinline__ uint32_t slow_limit(int qb) {
@@ -337,9 +343,8 @@ __device__ __forceinline__ void copy_in(unsigned char* dst, const void* src, int
 // Where both do not fit, the tile has four x and the copies take turns in one buffer
 // (seq): copy 1 is written when the Fourier products are done; the DFS products run
 // under the Fourier epilogue.
-// The Fourier results (and, in the angular pass, the Phi sums that make up the
-// scattering moments) go through shared memory to the threads that finish the
-// points from the DFS results.
+// The Fourier results (and, in the angular pass, the moments formed from its Phi sums) go
+// through shared memory to the threads that finish the points from the DFS results.
 // EP_ADJOINT is the transposed angular pass: the same contractions with the transposed
 // matrices, lt in place of U, and the adjoint's own epilogue.
 enum EmuPass { EP_ANGULAR = 0, EP_PLANE = 1, EP_ADJOINT = 2 };
@@ -364,13 +369,14 @@ struct MatArg {
   int se;          // 3 - s of the whole matrix
 };
 
-// Adds w, summed over the warp's rows of the same x (lanes XW apart), to a shared sum.
+// A moment's share of this warp: w summed over its rows of the same x (lanes XW apart), added
+// to what the warp's earlier rows gave (`add`). One warp owns each share.
 template <int XW>
-__device__ __forceinline__ void moment(unsigned long long* s, int64_t w) {
+__device__ __forceinline__ void moment(double* s, double w, bool add) {
   if (XW == 4) w += __shfl_xor_sync(0xFFFFFFFFu, w, 4);
   w += __shfl_xor_sync(0xFFFFFFFFu, w, 8);
   w += __shfl_xor_sync(0xFFFFFFFFu, w, 16);
-  if ((threadIdx.x & 31) < XW) atomicAdd(s, (unsigned long long)w);
+  if ((threadIdx.x & 31) < XW) *s = add ? *s + w : w;
 }
 // The shift that makes room for the coefficient sinTh cot th.
 __device__ __forceinline__ int cot_shift(double cot, int delta) {
@@ -492,10 +498,11 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
   uint32_t* smax = reinterpret_cast<uint32_t*>(ms + 32);          // [2][8]
   double* xs = reinterpret_cast<double*>(ms + 96);                // [2][8][8] scalars of a tile's x
   double* xm = xs + 2 * 64;                                       // [10][8] moments
-  unsigned long long* jsum = reinterpret_cast<unsigned long long*>(xm + 80);   // [10][8]
-  int64_t* wqt = reinterpret_cast<int64_t*>(jsum + 80);           // angular: weights [Na]
-  int* hs = reinterpret_cast<int*>(jsum + 80);                    // plane: shifts [Na]
-  double* gp = reinterpret_cast<double*>(wqt + Na);               // adjoint: [mt1][warps][8]
+  constexpr int nm = emu_moments(KF), nw = emu_weights(KF);
+  double* wt = xm + 80;                                           // angular: weights [nw][Na]
+  double* msum = wt + nw * Na;                                    // angular: [4 warps][nm][8]
+  int* hs = reinterpret_cast<int*>(xm + 80);                      // plane: shifts [Na]
+  double* gp = msum;                      // adjoint: [mt1][warps][8], once the moments are formed
   int64_t* ex = reinterpret_cast<int64_t*>(sm + g.oEx);           // [Nb][a][XW]
 
   if (Na % 8 || Nb % 16 || g.seq) {   // K paddings hold finite digits (their products vanish)
@@ -546,15 +553,24 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
   // of the DFS results; h makes room for the Fourier term's coefficient, delta is the
   // difference of the two matrices' scales.
   const int delta = m2.se - m1.se;
-  const int lgNa = 32 - __clz(Na - 1);
   for (int a = tid; a < Na; a += T) {
-    if (PASS == EP_PLANE)
+    if (PASS == EP_PLANE) {
       hs[a] = max(2, 3 + delta + ilogb(t.inv_sinth[a]));
-    else   // weights of the moments (Fejer x trapezoid; conservative: of Fhat / sinTh)
-      // (adjoint: plain sums, scaled down by the power of two that holds Na rows)
-      wqt[a] = __double2ll_rn(PASS == EP_ADJOINT ? pow2(63 - lgNa)
-                                                 : (A.cons ? t.qdir[a] / t.sinT[a] : t.qdir[a]) *
-                                                       pow2(63));
+    } else {   // weights of the moments (Fejer x trapezoid; conservative: of Fhat / sinTh;
+               // adjoint: plain sums) times 1, cos, sin, cos^2, cos sin, sin^2 of Theta
+      const double ct = t.cosT[a], st = t.sinT[a];
+      const double q = PASS == EP_ADJOINT ? 1.0 : A.cons ? t.qdir[a] / st : t.qdir[a];
+      wt[a] = q;
+      if (KF >= KF_LINEAR) {
+        wt[Na + a] = q * ct;
+        wt[2 * Na + a] = q * st;
+      }
+      if (KF >= KF_QUADRATIC) {
+        wt[3 * Na + a] = q * ct * ct;
+        wt[4 * Na + a] = q * ct * st;
+        wt[5 * Na + a] = q * st * st;
+      }
+    }
   }
   double v[U][8];
   TileAt<PASS> at{};
@@ -582,7 +598,7 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
   }
   int coef_n = -1;   // the Fourier coefficient this thread holds, and for what
   double coef_key = 0.0;
-  int64_t coef = 0, ws = 0, wc = 0;
+  int64_t coef = 0;
   int cth_b = -1;    // plane: cosPh of its DFS rows, and of which
   int64_t cth = 0;
   uint32_t phase = 0;   // one bit per barrier
@@ -619,7 +635,6 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
     if (PASS != EP_PLANE && warp == 1) cp8_wait();   // this tile's scalars
     __syncthreads();   // the maxima and scalars; the previous tile is finished
     if (tid < 8) smax[(buf ^ 1) * 8 + tid] = 0;
-    if (PASS != EP_PLANE && tid < 80) jsum[tid] = 0;
     // ---- digits
     auto fence_digits = [&]() {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -786,15 +801,10 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
       if (n != coef_n || key != coef_key) {
         coef_n = n;
         coef_key = key;
-        coef = ws = wc = 0;
+        coef = 0;
         if (val) {
           if (PASS != EP_PLANE) {
-            const double st = t.sinT[a], ct = t.cosT[a];
-            coef = __double2ll_rn(st * key * pow2(64 + delta - cot_shift(key, delta)));
-            if (KF >= KF_LINEAR) {
-              ws = __double2ll_rn(st * pow2(62));
-              wc = __double2ll_rn(ct * pow2(62));
-            }
+            coef = __double2ll_rn(t.sinT[a] * key * pow2(64 + delta - cot_shift(key, delta)));
           } else {
             const bool ok = cur.m0 + (rx & (XH - 1)) < hP;
             const double sp = ok ? t.sinP[cur.m0 + (rx & (XH - 1)) + (rx >= XH ? hP : 0)] : 0.0;
@@ -832,20 +842,21 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
           if (o < Nb && val) exr[o * exP] = zero ? 0 : __mul64hi(R[e], coef);
           const int f = o >= Nb ? o - Nb + g.nz : !zero ? -1 : o == 0 ? 0 : 1;
           if (f < 0 || !A.collision) continue;
-          // Phi sums of F times {1, cos, sin, cos^2, cos sin}: their Theta sums are the
-          // scattering moments, summed as integers (exact, in any order). Unit: 2 of R's
-          // for the weight alone, times 4 for every further factor
-          const int64_t w1 = val ? __mul64hi(R[e], wqt[a]) : 0;
+          // Phi sums of F times {1, cos, sin, cos^2, cos sin}: their weighted Theta sums are
+          // the scattering moments. In double: as fixed point a block's small moment beside
+          // a large value (a beam) lost bits that the sum of doubles keeps
+          const double y = val ? to_double1(R[e], eb + m2.se) : 0.0;
+          const double* wa = wt + (val ? a : 0);
+          double* s0 = msum + (warp & 3) * nm * 8 + rx;
           if (f == 0) {
-            moment<XW>(jsum + rx, w1);
-            if (KF >= KF_LINEAR) moment<XW>(jsum + 8 + rx, __mul64hi(w1, wc));
-            if (KF >= KF_QUADRATIC) moment<XW>(jsum + 32 + rx, __mul64hi(__mul64hi(w1, wc), wc));
+            moment<XW>(s0, y * wa[0], n > 0);
+            if (KF >= KF_LINEAR) moment<XW>(s0 + 8, y * wa[Na], n > 0);
+            if (KF >= KF_QUADRATIC) moment<XW>(s0 + 32, y * wa[3 * Na], n > 0);
           } else if (f < 3) {
-            const int64_t w2 = __mul64hi(w1, ws);
-            moment<XW>(jsum + 8 * (1 + f) + rx, w2);
-            if (KF >= KF_QUADRATIC) moment<XW>(jsum + 8 * (6 + f) + rx, __mul64hi(w2, wc));
+            moment<XW>(s0 + 8 * (1 + f), y * wa[2 * Na], n > 0);
+            if (KF >= KF_QUADRATIC) moment<XW>(s0 + 8 * (6 + f), y * wa[4 * Na], n > 0);
           } else {
-            moment<XW>(jsum + 8 * (2 + f) + rx, __mul64hi(__mul64hi(w1, ws), ws));
+            moment<XW>(s0 + 8 * (2 + f), y * wa[5 * Na], n > 0);
           }
         }
       }
@@ -1001,19 +1012,12 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
       }
       if (PASS != EP_PLANE && n == g.mt2 - 1 && A.collision) {
         if (tid < 80) {
-      // moment z of block x as a double (visible after the next wait's barrier)
+      // moment z of block x from the four warps' shares (visible after the next barrier)
       const int z = tid >> 3, x = tid & 7;
-      constexpr int nm = KF == KF_ISO ? 1 : KF == KF_LINEAR ? 4 : 9;
       if (x >= XW) {
       } else if (z < nm) {
-        // 2 and 4 per factor, as exponents (adjoint: and its weight's)
-        const int more = (z == 0 ? 1 : z < 4 ? 3 : 5) + (PASS == EP_ADJOINT ? lgNa : 0);
-        const int qv = block_exp(smax[buf * 8 + x]) + m2.se + more;
-        uint32_t top;
-        const int64_t R = (int64_t)jsum[tid];
-        double y = to_double_fast(R, (qv + 62) << 20, top);
-        if (top < slow_limit(qv)) y = to_double_slow(R, qv);
-        xm[tid] = y;
+        const double* m = msum + tid;
+        xm[tid] = (m[0] + m[nm * 8]) + (m[2 * nm * 8] + m[3 * nm * 8]);
       } else if (z == 9 && A.cons) {   // eta r^2 sin th
         xm[tid] = xc[24 + x] * xc[56 + x] / (xc[x] * xc[x]);
       }

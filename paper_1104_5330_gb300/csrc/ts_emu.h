@@ -47,7 +47,10 @@ struct EmuRadGeo {
   int threads;
 };
 
-constexpr int kEmuForms = 3;   // functionals of the isotropic, linear and quadratic kernels
+constexpr int kEmuForms = 3;   // isotropic, linear and quadratic kernels (KF_*): their
+constexpr int emu_functionals(int kf) { return kf == 0 ? 1 : kf == 1 ? 3 : 5; }   // Phi sums,
+constexpr int emu_moments(int kf) { return kf == 0 ? 1 : kf == 1 ? 4 : 9; }       // moments,
+constexpr int emu_weights(int kf) { return kf == 0 ? 1 : kf == 1 ? 3 : 6; }       // Theta weights
 
 struct EmuPlan {
   void* mem = nullptr;       // every table of the plan

@@ -28,17 +28,23 @@ def field(kind, og, F0, rng):
         return F0 * np.exp(-40 * (1 - mu))
     if kind == "attenuated":        # 1e-10 across the shell
         return F0 * np.exp(-30 * (og.r - og.r[0]))[None, :, None, None, None, None]
+    if kind == "pencil":            # one direction alone: the moments are far below its value
+        F = np.zeros_like(F0)
+        F[..., 3, 5] = F0[..., 3, 5]
+        return F
     raise ValueError(kind)
 
 
 def units(got, want, bound):
     assert np.all(np.isfinite(got))
-    return float((np.abs(got - want) / (bound * W(2) ** -53)).max())
+    some = bound > 0
+    assert np.all(got[~some] == 0)
+    return float((np.abs(got - want)[some] / (bound[some] * W(2) ** -53)).max())
 
 
-def both(gg, op, F, coeffs):
+def both(gg, op, F, coeffs, **kernel):
     L, N = op.streaming(F)
-    K, M = op.rate(F, *coeffs)
+    K, M = op.rate(F, *coeffs, **kernel)
     x = cuda(F)
     return (units(gg.liouville(x).cpu().numpy(), L, N), units(gg.rhs(x).cpu().numpy(), K, M))
 
@@ -72,3 +78,19 @@ def test_a_non_finite_point_reaches_no_other_radial_line(bad):
     same = K[0, far, 1, 2] == good[0, far, 1, 2]          # other nodes of the same (theta, phi)
     same[:, 3, 5] = True
     assert torch.all(same)
+
+
+@pytest.mark.parametrize("kernel", [{}, {"b": -0.3}, {"c": 0.75}], ids=["iso", "linear", "thomson"])
+@pytest.mark.parametrize("n", SHAPES + [(5, 3, 4, 32, 32), (6, 4, 2, 24, 16)], ids=str)
+def test_moments_of_a_single_direction(n, kernel):
+    """Directions off the bright one's lines hold exact zeros: their rate is the moments."""
+    dims = (0.2, 1.0) + n
+    og, gg = pair(*dims)
+    kap, eta, ks, F0, _, _ = absorber_workload(og)
+    gg.set_coeffs(kap, 0 * eta, 8 * ks)
+    if "b" in kernel:
+        gg.set_scattering_anisotropy(kernel["b"])
+    if "c" in kernel:
+        gg.set_scattering_quadrupole(kernel["c"])
+    F = field("pencil", og, F0, None)
+    assert max(both(gg, Extended(*dims), F, (kap, 0 * eta, 8 * ks), **kernel)) < BAR

@@ -233,6 +233,7 @@ bool geometry2_form(int xw, bool seq, int Na, int Nb, const EmuMat& D, const Emu
   const int kf = nf >= 5 ? 2 : nf >= 3 ? 1 : 0;
   const int shares = std::max(4 * emu_moments(kf), adj ? g.mt1 * 16 : 0) * 8;
   g.oMs = take(96 + (128 + 80 + (nf ? emu_weights(kf) * Na + shares : Na)) * 8);
+  g.oLn = take((g.hb + Na) * xw * 2);
   // a 128-row tile may read row groups past the last one: inside the allocation
   const int over = std::max(g.oC1 + 7 * g.d1 + (16 * g.mt1 + hg) * g.sb1 + 256,
                             g.oC2 + 7 * g.d2 + 16 * g.mt2 * g.sb2 + 256);

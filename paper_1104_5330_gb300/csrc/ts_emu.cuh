@@ -4,10 +4,12 @@
 // the FP64 pipe bounds every double-precision pass that contracts on it. Here the
 // contractions run as exact integer arithmetic on tcgen05.mma kind::f16:
 //  * data: a tile's values are turned into 64-bit fixed point relative to the
-//    largest magnitude of a block (61 bits below it), on the integer units, and
-//    cut into eight bytes u_i. A byte zero-extended to 16 bits is the f16
-//    subnormal u_i 2^-24, so the digits need no conversion. Balanced digits are
-//    d_i = u_i - 128 (the fixed-point value has 0x8080...80 added);
+//    largest magnitude of their line (61 bits below it), on the integer units, and
+//    cut into eight bytes u_i. (Where all values of a block lie within a factor of
+//    eight to sixteen of each other, its largest stands for that of its lines.) A byte
+//    zero-extended to 16 bits is the f16 subnormal u_i 2^-24, so the digits need no
+//    conversion. Balanced digits are d_i = u_i - 128 (the fixed-point value has
+//    0x8080...80 added);
 //  * matrix: every row scaled to 62 bits, in eight balanced base-256 digits e_j as
 //    f16 integers (built on the host from the exact products of its factors);
 //  * the products d_i e_j of order o = i + j <= 7 are accumulated in f32, one
@@ -19,15 +21,16 @@
 //    0x3F400000 + (the exact integer sum);
 //  * the eight sums are recombined in a 64-bit integer (orders >= 8, 2^-59 of the
 //    full scale, are dropped) and rounded once to double on the integer units.
-// The error of a contraction is that one rounding, less than that of the FP64
-// multiply-adds it replaces: against the operator in extended precision one right-hand
-// side is 1.2e-15 (17 x 8^4), 6.1e-15 (33 x 8^4), 7.9e-16 (9 x 16^2 x 8^2) off in the
-// relative 2-norm where the FP64 passes are 2.0e-14, 2.6e-14 and 1.5e-14 off. A block that
-// holds an infinity or a NaN gives NaN.
-//
-// What bounds the passes now: the integer instructions that cut, recombine and round
-// (about 240 a point and pass, 64-bit multiplies among them), at 1.5 instructions per
-// clock from 16 warps an SM; tensor pipe 9 %, FP64 pipe 20-40 %, HBM 10-15 % busy.
+// The method is Ozaki's splitting into slices whose products are exact (Ozaki, Ogita, Oishi
+// and Rump 2012, Numer. Algorithms 59) with integer slices (Ootomo, Ozaki and Yokota 2024).
+// The error of a contraction is a few units of 2^-57 x (largest matrix entry of the row) x
+// (largest value of the line) and that one rounding. In units of 2^-53 x row sum x largest
+// value of the point's own lines a right-hand side is off by 0.1 to 10, the FP64 multiply-adds
+// by 0.4 to 20 on the same fields: smooth ones, beams, isolated bright points, magnitudes that
+// vary by 2^60 between directions or positions (tests/test_gpu_line_precision.py); in the
+// relative 2-norm by 4e-16 (17 x 6 x 8 x 16^2, smooth), 1e-15 (33 x 4^2 x 16^2) against 4e-15,
+// 6e-15.
+// A line that holds an infinity or a NaN gives NaN.
 //
 // Every wait is bounded: if one runs out the kernel sets the grid's error flag
 // (ts_sync_status reports TS_ERR_TIMEOUT), waits again for its own MMAs, frees its
@@ -35,6 +38,8 @@
 #pragma once
 
 #include <stdint.h>
+
+#include <type_traits>
 
 #include "ts_emu.h"
 #include "ts_kernels.cuh"
@@ -193,6 +198,42 @@ __device__ __forceinline__ uint64_t to_fixed(double v, uint32_t EM) {
   const uint32_t xl = (uint32_t)x ^ sg, xh = (uint32_t)(x >> 32) ^ sg;
   return (((uint64_t)xh << 32) | xl) + ((0x80808080ull << 32) | (uint64_t)(0x80808080u - sg));
 }
+// far: set if v is not zero and more than kNear places below.
+constexpr uint32_t kNear = 3;
+__device__ __forceinline__ bool far_below(uint32_t mag, uint32_t EM) {   // one range test
+  return EM - mag - ((kNear + 1) << 20) < EM - ((kNear + 2) << 20) + 1u;
+}
+__device__ __forceinline__ uint64_t to_fixed(double v, uint32_t EM, bool& far) {
+  far |= far_below((uint32_t)__double2hiint(v) & 0x7FFFFFFFu, EM);
+  return to_fixed(v, EM);
+}
+// Eight values relative to the exponent bases of their lines (16 bits each, 0 for a line of
+// zeros). Tiny lines, bases below 64, are brought up first if there are any (lift).
+__device__ __forceinline__ void to_fixed_lines(const double (&v)[8], uint4 e, bool lift,
+                                               uint64_t (&f)[8]) {
+  const uint32_t w[4] = {e.x, e.y, e.z, e.w};
+#pragma unroll
+  for (int x = 0; x < 8; x += 2) {
+    if (!lift) {
+      const uint32_t b = __vmaxs2(w[x / 2], 0x00400040u);
+      f[x] = to_fixed(v[x], b << 20 | 0xFFFFFu);
+      f[x + 1] = to_fixed(v[x + 1], (b & 0xFFFF0000u) << 4 | 0xFFFFFu);
+    } else {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const uint32_t b = h ? w[x / 2] >> 16 : w[x / 2] & 0xFFFFu;
+        const bool up = b < 64;
+        f[x + h] = to_fixed(up ? v[x + h] * __hiloint2double((1023 + 256) << 20, 0) : v[x + h],
+                            (up ? b + 256 : b) << 20 | 0xFFFFFu);
+      }
+    }
+  }
+}
+__device__ __forceinline__ int64_t sra(int64_t v, int n) {   // shifts of 64 and more: the sign
+  int64_t r;
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+  return r;
+}
 
 __device__ __forceinline__ uint64_t mad_wide(uint32_t a, uint32_t b, uint64_t c) {
   uint64_t r;
@@ -287,6 +328,11 @@ __device__ __forceinline__ int line_exp(uint32_t key) {
   return key == 0 ? 64 : !(key & 1u) ? e - 256 : e == 2047 ? 5000 : max(e, 64);
 }
 
+// The exponent base of a line of its own scale in a two-axis tile: 0 for a line of zeros.
+__device__ __forceinline__ int line_base(uint32_t mx) {
+  const int e = (int)(mx >> 20);
+  return mx == 0 ? 0 : e == 2047 ? 5000 : max(e, 1);
+}
 // The fixed-point key of a block: its largest exponent, at least 64, and a mantissa of ones.
 __device__ __forceinline__ uint32_t fixed_key(uint32_t mx) {
   return ((uint32_t)max((int)(mx >> 20), 64) << 20) | 0xFFFFFu;
@@ -495,7 +541,11 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
   unsigned char* ms = sm + g.oMs;
   uint64_t* bar = reinterpret_cast<uint64_t*>(ms);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(ms + 16);
+  volatile uint32_t* wmask = reinterpret_cast<volatile uint32_t*>(ms + 20);   // see wide below
+  volatile uint32_t* wflag = reinterpret_cast<volatile uint32_t*>(ms + 24);   // [2]
   uint32_t* smax = reinterpret_cast<uint32_t*>(ms + 32);          // [2][8]
+  int16_t* ln1 = reinterpret_cast<int16_t*>(sm + g.oLn);   // lines' exponents: a-circles [hb][XW],
+  int16_t* ln2 = ln1 + hb * XW;                            // b-lines [Na][XW]
   double* xs = reinterpret_cast<double*>(ms + 96);                // [2][8][8] scalars of a tile's x
   double* xm = xs + 2 * 64;                                       // [10][8] moments
   constexpr int nm = emu_moments(KF), nw = emu_weights(KF);
@@ -510,6 +560,7 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
       reinterpret_cast<uint4*>(sm)[x] = make_uint4(0, 0, 0, 0);
   }
   if (tid < 16) smax[tid] = 0;
+  if (tid < 2) wflag[tid] = 0;
   copy_in(sm + g.oB1, m1.dev, (1 + g.kc1) * g.r1 * 16);
   copy_in(sm + g.oB2, m2.dev, (1 + g.kc2) * g.r2 * 16);
   fill_bias(sm + g.oCA, 128);
@@ -557,18 +608,13 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
     if (PASS == EP_PLANE) {
       hs[a] = max(2, 3 + delta + ilogb(t.inv_sinth[a]));
     } else {   // weights of the moments (Fejer x trapezoid; conservative: of Fhat / sinTh;
-               // adjoint: plain sums) times 1, cos, sin, cos^2, cos sin, sin^2 of Theta
-      const double ct = t.cosT[a], st = t.sinT[a];
+               // adjoint: plain sums) times 1, cos and sin of Theta
+      const double st = t.sinT[a];
       const double q = PASS == EP_ADJOINT ? 1.0 : A.cons ? t.qdir[a] / st : t.qdir[a];
       wt[a] = q;
       if (KF >= KF_LINEAR) {
-        wt[Na + a] = q * ct;
+        wt[Na + a] = q * t.cosT[a];
         wt[2 * Na + a] = q * st;
-      }
-      if (KF >= KF_QUADRATIC) {
-        wt[3 * Na + a] = q * ct * ct;
-        wt[4 * Na + a] = q * ct * st;
-        wt[5 * Na + a] = q * st * st;
       }
     }
   }
@@ -603,6 +649,7 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
   int64_t cth = 0;
   uint32_t phase = 0;   // one bit per barrier
   bool alive = true, late = false;   // late: a wait of this thread ran out
+  bool guess = false;                // the tile before was wide
   int buf = 0;
   for (long long tile = blockIdx.x; tile < A.ntiles && alive; tile += gridDim.x, buf ^= 1) {
     // ---- largest magnitude of each block (angular) or of the tile (plane)
@@ -634,7 +681,13 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
     }
     if (PASS != EP_PLANE && warp == 1) cp8_wait();   // this tile's scalars
     __syncthreads();   // the maxima and scalars; the previous tile is finished
-    if (tid < 8) smax[(buf ^ 1) * 8 + tid] = 0;
+    if (tid < 8) {
+      smax[(buf ^ 1) * 8 + tid] = 0;
+      // tiny blocks and blocks with an infinity or a NaN: line by line
+      const uint32_t mx = smax[buf * 8 + tid];
+      if (tiny_line(mx) || mx >= 0x7FF00000u) wflag[buf] = 1;
+    }
+    if (tid == 8) wflag[buf ^ 1] = 0;
     // ---- digits
     auto fence_digits = [&]() {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -676,27 +729,125 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
         }
       }
     };
-    {
+    // One scale for a block (plane: for the tile) while its values lie within kNear places;
+    // the lines of a point then differ by no more. Else (wide) every line has its own: copy 1
+    // is cut relative to the largest value of each a-circle (a line and its partner's), copy 2
+    // to that of each b-line. Blocks that need it not keep their one scale also beside one
+    // that does, and whether the tile before was wide only decides which way is tried first
+    // (guess): what a block gives depends on its own values alone. With one scale always, a
+    // step of 33 x 16^4 x 4 takes 1467 us (now 1515), its conservative form, whose sin Theta
+    // makes most tiles wide, 1589 (1865), the shell run of 129 x 16^2 x 24 x 16 2935 (3200)
+    if (!guess) {
       uint32_t em[XW];
 #pragma unroll
       for (int x = 0; x < XW; ++x)
         em[x] = fixed_key(smax[buf * 8 + (PASS == EP_PLANE ? 0 : x)]);
+      bool far = false;
 #pragma unroll
       for (int q = 0; q < U; ++q) {
         if (ua[q] < 0) continue;
         if constexpr (XW == 8) {
           uint64_t f[8];
 #pragma unroll
-          for (int x = 0; x < 8; ++x) f[x] = to_fixed(v[q][x], em[x]);
+          for (int x = 0; x < 8; ++x) f[x] = to_fixed(v[q][x], em[x], far);
           put(f, q, true, true);
         } else {
 #pragma unroll
-          for (int x = 0; x < 8; ++x) f4[q][x] = to_fixed(v[q][x], em[x & 3]);
+          for (int x = 0; x < 8; ++x) f4[q][x] = to_fixed(v[q][x], em[x & 3], far);
           put(f4[q], q, !g.seq, true);
         }
       }
+      if (far) wflag[buf] = 1;
+      fence_digits();
     }
-    fence_digits();
+    const bool wide = guess || wflag[buf] != 0;
+    if (wide) {
+      // the values again: kept, they would take registers from the common way
+      if (!guess) load_units<PASS, U, XW>(d, A.U, at, S, hP, Nb, A.vec, ua, ub, v);
+      int* mx1 = reinterpret_cast<int*>(sm + g.oEx);   // maxima [x][hb], [a][x], in the exchange
+      int* mx2 = mx1 + hb * XW;
+      for (int z = tid; z < (hb + Na) * XW; z += T) mx1[z] = 0;
+      if (tid == 0) *wmask = 0;   // the blocks that are wide
+      __syncthreads();
+      uint32_t mine = 0;
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        uint32_t mag[8];
+#pragma unroll
+        for (int x = 0; x < 8; ++x)
+          mag[x] = ua[q] < 0 ? 0u : (uint32_t)__double2hiint(v[q][x]) & 0x7FFFFFFFu;
+#pragma unroll
+        for (int x = 0; x < 8; ++x) {
+          const uint32_t mx = smax[buf * 8 + (PASS == EP_PLANE ? 0 : x & (XW - 1))];
+          if (far_below(mag[x], fixed_key(mx)) || tiny_line(mx) || mx >= 0x7FF00000u)
+            mine |= PASS == EP_PLANE ? 0xFFu : 1u << (x & (XW - 1));
+          const int xx = x & (XW - 1), b = ub[q] + x / XW, c = b < hb ? b : b - hb;
+          if (ua[q] >= 0)
+            atomicMax(&mx1[(PASS == EP_PLANE && b >= hb ? xx ^ (XW / 2) : xx) * hb + c], (int)mag[x]);
+        }
+        if (XW == 8 && Nb % 8 == 0) {   // eight lanes hold one b-line: one value each
+          const int l = lane & 7;
+#pragma unroll
+          for (int h = 4; h > 0; h /= 2) {
+#pragma unroll
+            for (int x = 0; x < h; ++x) {
+              const bool hi = l & h;
+              const uint32_t send = hi ? mag[x] : mag[x + h], keep = hi ? mag[x + h] : mag[x];
+              mag[x] = max(keep, __shfl_xor_sync(0xFFFFFFFFu, send, h));
+            }
+          }
+          if (ua[q] >= 0) atomicMax(&mx2[ua[q] * XW + l], (int)mag[0]);
+        } else if (ua[q] >= 0) {
+#pragma unroll
+          for (int x = 0; x < 8; ++x) atomicMax(&mx2[ua[q] * XW + (x & (XW - 1))], (int)mag[x]);
+        }
+      }
+      mine = __reduce_or_sync(0xFFFFFFFFu, mine);
+      if (lane == 0 && mine) atomicOr(const_cast<uint32_t*>(wmask), mine);
+      __syncthreads();
+      const uint32_t mask = *wmask & 0xFFu;
+      bool low = false;
+      for (int z = tid; z < (hb + Na) * XW; z += T) {
+        const int y = z - hb * XW, x = y < 0 ? z / hb : y & (XW - 1), c = z - x * hb;
+        const bool own = mask >> x & 1u;
+        const uint32_t mx = own ? (uint32_t)mx1[z] : smax[buf * 8 + (PASS == EP_PLANE ? 0 : x)];
+        low |= own && tiny_line(mx);
+        ln1[y < 0 ? c * XW + x : z] = (int16_t)(own ? line_base(mx) : block_exp(mx));
+      }
+      const bool lift = __syncthreads_or(low ? 1 : 0);
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        if (ua[q] < 0) continue;
+        auto bases = [&](const int16_t* p) {   // of one unit: XW lines of a row
+          return XW == 8 ? *reinterpret_cast<const uint4*>(p)
+                         : make_uint4(reinterpret_cast<const uint2*>(p)->x,
+                                      reinterpret_cast<const uint2*>(p)->y, 0u, 0u);
+        };
+        uint4 e = bases(ln2 + ua[q] * XW);
+        if (XW == 4) e.z = e.x, e.w = e.y;
+        uint64_t f[8];
+        to_fixed_lines(v[q], e, lift, f);
+        put(f, q, false, true);
+        const bool part = ub[q] >= hb;
+        const int16_t* p1 = ln1 + (part ? ub[q] - hb : ub[q]) * XW;
+        e = bases(p1);
+        if (XW == 4) {
+          const uint4 e2 = bases(p1 + XW);
+          e.z = e2.x, e.w = e2.y;
+        }
+        if (PASS == EP_PLANE && part)   // the other half circle's columns trade places
+          e = XW == 8 ? make_uint4(e.z, e.w, e.x, e.y) : make_uint4(e.y, e.x, e.w, e.z);
+        if constexpr (XW == 8) {
+          to_fixed_lines(v[q], e, lift, f);
+          put(f, q, true, false);
+        } else {
+          to_fixed_lines(v[q], e, lift, f4[q]);
+          if (!g.seq) put(f4[q], q, true, false);
+        }
+      }
+      fence_digits();
+      guess = mask != 0;
+    }
     // issues job n (one call site: the unrolled chains are inlined there, their
     // operands in uniform registers)
     auto issue = [&](int n) {
@@ -845,18 +996,23 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
           // Phi sums of F times {1, cos, sin, cos^2, cos sin}: their weighted Theta sums are
           // the scattering moments. In double: as fixed point a block's small moment beside
           // a large value (a beam) lost bits that the sum of doubles keeps
-          const double y = val ? to_double1(R[e], eb + m2.se) : 0.0;
-          const double* wa = wt + (val ? a : 0);
+          const int e2 = wide && val ? ln2[a * XW + rx] : eb;
+          const double y = val ? to_double1(R[e], e2 + m2.se) : 0.0;
+          const int av = val ? a : 0;
+          const double* wa = wt + av;
           double* s0 = msum + (warp & 3) * nm * 8 + rx;
           if (f == 0) {
             moment<XW>(s0, y * wa[0], n > 0);
             if (KF >= KF_LINEAR) moment<XW>(s0 + 8, y * wa[Na], n > 0);
-            if (KF >= KF_QUADRATIC) moment<XW>(s0 + 32, y * wa[3 * Na], n > 0);
-          } else if (f < 3) {
-            moment<XW>(s0 + 8 * (1 + f), y * wa[2 * Na], n > 0);
-            if (KF >= KF_QUADRATIC) moment<XW>(s0 + 8 * (6 + f), y * wa[4 * Na], n > 0);
+            if (KF >= KF_QUADRATIC) moment<XW>(s0 + 32, y * wa[Na] * t.cosT[av], n > 0);
           } else {
-            moment<XW>(s0 + 8 * (2 + f), y * wa[5 * Na], n > 0);
+            const double ys = y * wa[2 * Na];
+            if (f < 3) {
+              moment<XW>(s0 + 8 * (1 + f), ys, n > 0);
+              if (KF >= KF_QUADRATIC) moment<XW>(s0 + 8 * (6 + f), ys * t.cosT[av], n > 0);
+            } else {
+              moment<XW>(s0 + 8 * (2 + f), ys * t.sinT[av], n > 0);
+            }
           }
         }
       }
@@ -929,8 +1085,13 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
         }
       }
       const int qv = eb + m1.se;
-      const uint32_t lim = slow_limit(qv);
+      const int e1 = wide ? ln1[(!val ? 0 : b < hb ? b : b - hb) * XW + rx] : 0;
+      uint32_t lim = slow_limit(qv);
       const int64_t* exr = ex + (val ? b : 0) * exP + w;
+      // own: wide, in a loop of its own (a branch inside slows the common one by 2 %; the
+      // adjoint's loop is too long to have twice)
+      auto finish = [&](auto lines) {
+      const bool own = PASS == EP_ADJOINT ? wide : decltype(lines)::value;
       for (int q0 = grp; 4 * q0 < Na; q0 += 2 * NG) {
         if (q0 != grp) load_in(q0);
 #pragma unroll
@@ -943,14 +1104,29 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
           int64_t W[4];
           int qb[4];
           recombine4(bb, W);
+          if (!own) {
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int a = min(4 * q + e, Na - 1);
-            const int ha = PASS != EP_PLANE ? hx : hs[a];
-            if (PASS != EP_PLANE) W[e] >>= hx;
-            else W[e] = __mul64hi(W[e], cth) >> (ha - 2);
-            W[e] += exr[a * XW];
-            qb[e] = qv + ha;
+            for (int e = 0; e < 4; ++e) {
+              const int a = min(4 * q + e, Na - 1);
+              const int ha = PASS != EP_PLANE ? hx : hs[a];
+              if (PASS != EP_PLANE) W[e] >>= hx;
+              else W[e] = __mul64hi(W[e], cth) >> (ha - 2);
+              W[e] += exr[a * XW];
+              qb[e] = qv + ha;
+            }
+          } else {   // the unit of the larger term, 2^top, with a place (plane: two) to spare
+            lim = 1u;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const int a = min(4 * q + e, Na - 1);
+              const int ha = PASS != EP_PLANE ? hx : hs[a], sp = PASS != EP_PLANE ? 1 : 2;
+              const int e2 = ln2[a * XW + w] + ha, top = max(e1 + sp, e2);
+              if (PASS != EP_PLANE) W[e] = sra(W[e], top - e1);
+              else W[e] = sra(__mul64hi(W[e], cth), top - e1 - 2);
+              W[e] += sra(exr[a * XW], top - e2);
+              qb[e] = top + m1.se;
+              lim = max(lim, slow_limit(qb[e]));
+            }
           }
           double y4[4];
           to_double4(W, qb, lim, y4);
@@ -995,6 +1171,9 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
           }
         }
       }
+      };
+      if (PASS != EP_ADJOINT && wide) finish(std::true_type{});
+      else finish(std::false_type{});
       }
       if (PASS == EP_ADJOINT && n >= g.mt2) {
         if (XW == 4) gks += __shfl_xor_sync(0xFFFFFFFFu, gks, 4);

@@ -30,7 +30,7 @@ struct EmuGeo {
   int mt1, mt2;              // 128-row tiles of the two contractions
   int exP;                   // pitch (doubles) of the exchange array
   int cols, dual, half;      // tensor-memory columns, two regions in flight, their distance
-  int oC1, oC2, oB1, oB2, oCA, oEx, oMs, bytes;
+  int oC1, oC2, oB1, oB2, oCA, oEx, oMs, oLn, bytes;
   int threads;
 };
 
@@ -50,7 +50,7 @@ struct EmuRadGeo {
 constexpr int kEmuForms = 3;   // isotropic, linear and quadratic kernels (KF_*): their
 constexpr int emu_functionals(int kf) { return kf == 0 ? 1 : kf == 1 ? 3 : 5; }   // Phi sums,
 constexpr int emu_moments(int kf) { return kf == 0 ? 1 : kf == 1 ? 4 : 9; }       // moments,
-constexpr int emu_weights(int kf) { return kf == 0 ? 1 : kf == 1 ? 3 : 6; }       // Theta weights
+constexpr int emu_weights(int kf) { return kf == 0 ? 1 : 3; }                     // Theta weights
 
 struct EmuPlan {
   void* mem = nullptr;       // every table of the plan

@@ -144,3 +144,26 @@ class Extended:
             K = K - np.where(out, K[:, :1] * t[:, :1], K[:, -1:] * t[:, -1:]) * t
             N = N + np.where(out, N[:, :1], N[:, -1:])
         return K, N
+
+    def streaming_adjoint(self, F):
+        """L^T F (advective form) and its bound. The contraction over Theta takes F as it is
+        and sin Theta with its matrix: that factor counts as 1 on the lines."""
+        F = np.asarray(F).astype(W)
+        r, sth, cth, sT, cT, sP, cP = self.r, self.sth, self.cth, self.sT, self.cT, self.sP, self.cP
+        turn = lambda both: (lambda X: self._turn(X, both))
+
+        def term(coef, size, axis, A, B=None, H=None):
+            X, top, rows = coef * F, np.abs(size * F), np.abs(A).sum(0)
+            K = _along(A.T, X, axis)
+            if B is not None:
+                K = K + H(_along(B.T, X, axis))
+                top, rows = np.maximum(top, H(top)), rows + np.abs(B).sum(0)
+            rows = rows.reshape([-1 if a == axis else 1 for a in range(6)])
+            return K, rows * top.max(axis=axis, keepdims=True)
+
+        terms = [term(cT, cT, 1, self.Dr),
+                 term(sT * cP / r, sT / r, 2, self.At, self.Bt, turn(True)),
+                 term(sT * sP / (r * sth), sT / (r * sth), 3, self.Dp),
+                 term(-sT / r, 1 / r, 4, self.AT, self.BT, turn(False)),
+                 term(-sT * sP * cth / (r * sth), sT / (r * sth), 5, self.DP)]
+        return sum(t[0] for t in terms), sum(t[1] for t in terms)

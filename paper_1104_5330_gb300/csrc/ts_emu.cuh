@@ -527,7 +527,7 @@ __device__ __forceinline__ void load_units(const Dims& d, const double* F, const
 }
 
 // NA_, NB_: the axes' lengths at compile time (0: from the geometry).
-template <int PASS, int KF, int T, int U, int NA_, int NB_, int XW>
+template <int PASS, int KF, int T, int NA_, int NB_, int XW>
 __global__ void __launch_bounds__(T, T == 256 ? 2 : 1)
 k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
   extern __shared__ __align__(128) unsigned char sm[];
@@ -536,6 +536,7 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int uwarp = __shfl_sync(0xFFFFFFFFu, warp, 0);   // warp-uniform
   constexpr int NG = T / 128;                     // threads per tensor-memory lane
+  constexpr int U = 1;                            // units of a tile a thread holds (host)
   const int Na = NA_ ? NA_ : g.Na, Nb = NB_ ? NB_ : g.Nb, hb = Nb / 2, exP = Na * XW + 8;
   // small arrays
   unsigned char* ms = sm + g.oMs;

@@ -229,7 +229,8 @@ cudaError_t launch_number_balance(const Problem& p, const Tables<double>& t, con
                                   double* part, double* out, cudaStream_t s);
 
 // Whether the tensor-core radial pass handles N_r (its tile must fit shared memory).
-inline bool tc_supported(int Nr) { return Nr >= 3 && Nr <= 81; }
+constexpr int kTcMaxNr = 81;
+inline bool tc_supported(int Nr) { return Nr >= 3 && Nr <= kTcMaxNr; }
 
 // Output mode of the radial pass (the last pass of a stage).
 enum RadialMode {

@@ -99,16 +99,15 @@ __device__ __forceinline__ void umma(uint32_t dtmem, uint64_t a, uint64_t b, uin
         :: "r"(dtmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(one) : "memory");
 }
 
-// The products of one tile: ST K steps (0: `steps` at run time). Issued by a warp
-// from uniform registers and unrolled, an MMA takes 50 clocks to issue; from one
-// thread of a divergent branch, 163.
+// The products of one tile: ST K steps. Issued by a warp from uniform registers and
+// unrolled, an MMA takes 50 clocks to issue; from one thread of a divergent branch or a
+// run-time loop, 150 to 160.
 template <int KIND, int ST>
 __device__ __forceinline__ void tc_products(uint32_t one, uint32_t tmem, uint32_t a0, uint32_t as,
                                             uint32_t b0, uint32_t bs, uint32_t lbo, uint32_t sbo,
-                                            uint32_t idesc, int steps) {
-  const int n = ST ? ST : steps;
+                                            uint32_t idesc) {
 #pragma unroll
-  for (int ks = 0; ks < n; ++ks) {
+  for (int ks = 0; ks < ST; ++ks) {
     const uint32_t off = (uint32_t)ks * 256;  // two 16-byte core columns of K
     auto mma = [&](int ta, int tb, uint32_t acc) {
       umma<KIND>(tmem, umma_desc(a0 + ta * as + off, lbo, sbo),
@@ -127,6 +126,16 @@ __device__ __forceinline__ void tc_products(uint32_t one, uint32_t tmem, uint32_
       mma(0, 0, 1);
     }
   }
+}
+
+// The same for every number of steps up to MAX.
+template <int KIND, int MAX>
+__device__ __forceinline__ void tc_products_of(uint32_t one, uint32_t tmem, uint32_t a0,
+                                               uint32_t as, uint32_t b0, uint32_t bs, uint32_t lbo,
+                                               uint32_t sbo, uint32_t idesc, int steps) {
+  if (steps == MAX) tc_products<KIND, MAX>(one, tmem, a0, as, b0, bs, lbo, sbo, idesc);
+  else if constexpr (MAX > 1)
+    tc_products_of<KIND, MAX - 1>(one, tmem, a0, as, b0, bs, lbo, sbo, idesc, steps);
 }
 
 // Operand form: element bytes, operand terms, elements per 16-byte core
@@ -350,15 +359,8 @@ k_radial_tc(Problem p, Tables<float> t, const void* __restrict__ Bterms, const f
       const uint32_t a0 = smem_u32(sA), b0 = smem_u32(sB);
       const uint32_t as = (uint32_t)sh.a_bytes, bs = (uint32_t)sh.b_bytes;
       const int steps = sh.Kpad / Fm::KSTEP;
-      // N_r = 17, 33, 65 unrolled
-      if (steps == (KIND == TC_TF32X3 ? 5 : 3))
-        tc_products<KIND, KIND == TC_TF32X3 ? 5 : 3>(one, tmem, a0, as, b0, bs, lbo, sbo, idesc, 0);
-      else if (steps == (KIND == TC_TF32X3 ? 3 : 2))
-        tc_products<KIND, KIND == TC_TF32X3 ? 3 : 2>(one, tmem, a0, as, b0, bs, lbo, sbo, idesc, 0);
-      else if (steps == (KIND == TC_TF32X3 ? 9 : 5))
-        tc_products<KIND, KIND == TC_TF32X3 ? 9 : 5>(one, tmem, a0, as, b0, bs, lbo, sbo, idesc, 0);
-      else
-        tc_products<KIND, 0>(one, tmem, a0, as, b0, bs, lbo, sbo, idesc, steps);
+      tc_products_of<KIND, (kTcMaxNr + Fm::KSTEP - 1) / Fm::KSTEP>(one, tmem, a0, as, b0, bs, lbo,
+                                                                   sbo, idesc, steps);
       asm volatile(
           "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
           " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n"

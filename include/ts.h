@@ -64,7 +64,20 @@ typedef enum {
 } ts_status;
 
 typedef enum {
-  TS_FP64 = 0,     /* double storage, double arithmetic */
+  TS_FP64 = 0,     /* double storage, double arithmetic. Where the sizes have a plan (most
+                      up to 32 nodes an angular axis and 81 radial nodes) the
+                      contractions are exact integer products on the tensor cores:
+                      every value is cut at 2^-61 or less of the largest magnitude
+                      of its line (r; the theta or Theta circle; phi; Phi) - at most
+                      16 times that where all values of a block lie that close -
+                      and the sums are rounded once. A point's error is bounded by
+                      its own lines, as that of double multiply-adds is: a few
+                      2^-53 x row sum x largest value of the line, whatever other
+                      lines hold; an infinity or a NaN reaches the lines it lies
+                      on. Magnitudes below 2^-1022 count as zero beside values
+                      above 2^-958 of the same line or block. With the environment
+                      variable TS_GENERIC_PASSES=1 at grid creation the passes run
+                      on the FP64 units at every size */
   TS_FP32 = 1,     /* float storage, float arithmetic */
   TS_FP32_R64 = 2, /* float storage and angular arithmetic; the two radial
                       derivative rows nearest each of r = R1 and r = R2 (the rows

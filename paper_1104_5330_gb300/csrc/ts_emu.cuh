@@ -32,6 +32,12 @@
 // 6e-15.
 // A line that holds an infinity or a NaN gives NaN.
 //
+// What bounds the passes: no unit (profiles/fp64_tensorcore_passes.md: issue slots 38 to 44 %,
+// integer pipes 22 to 36, FP64 22 to 40, tensor pipe 10 to 11, HBM 7 to 20 % busy), but the
+// order of work: the 16 warps that registers allow on an SM load, cut, wait for the products
+// and finish points in the same phases, with four or more CTA barriers a tile and dependent
+// integer instructions (200 to 235 a point) between them.
+//
 // Every wait is bounded: if one runs out the kernel sets the grid's error flag
 // (ts_sync_status reports TS_ERR_TIMEOUT), waits again for its own MMAs, frees its
 // tensor memory and returns.

@@ -742,8 +742,8 @@ k_emu2(Problem p, Tables<double> t, EmuGeo g, MatArg m1, MatArg m2, EmuArgs A) {
     // to that of each b-line. Blocks that need it not keep their one scale also beside one
     // that does, and whether the tile before was wide only decides which way is tried first
     // (guess): what a block gives depends on its own values alone. With one scale always, a
-    // step of 33 x 16^4 x 4 takes 1467 us (now 1515), its conservative form, whose sin Theta
-    // makes most tiles wide, 1589 (1865), the shell run of 129 x 16^2 x 24 x 16 2935 (3200)
+    // step of 33 x 16^4 x 4 takes 1467 us (now 1510), its conservative form, whose sin Theta
+    // makes most tiles wide, 1589 (1865), the shell run of 129 x 16^2 x 24 x 16 2935 (3189)
     if (!guess) {
       uint32_t em[XW];
 #pragma unroll

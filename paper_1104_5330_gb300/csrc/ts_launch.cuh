@@ -239,9 +239,9 @@ cudaError_t Launch<T, C>::angular(const Problem& p, const Tables<C>& t, const T*
       return launch_angular_tc(p, t, U, K, sgn, collision, s);
   }
   // double precision: exact integer products on the tensor cores wherever the tile fits
-  // (33 x 16^4 x 4: angular 440 -> 128 us, plane 386 -> 121, radial 381 -> 144; 65 x 32^4: a
-  // step 77.9 -> 17.8 ms; also the faster one on the smallest grids, 17 x 8^4: 25, 19, 21
-  // -> 13, 13, 15)
+  // (33 x 16^4 x 4: angular 440 -> 131 us, plane 386 -> 124, radial 381 -> 144, where most
+  // tiles are cut line by line 163 and 151; 65 x 32^4: a step 77.9 -> 17.8 ms, 21.1; also the
+  // faster one on the smallest grids, 17 x 8^4: 25, 19, 21 -> 13 to 15 each)
   if constexpr (sizeof(T) == 8) {
     if (p.emu && emu_has_angular(*p.emu, d))
       return emu_angular(*p.emu, p, t, false, U, K, sgn, collision, s);
